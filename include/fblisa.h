@@ -190,12 +190,12 @@ FBL_API fbl_status geometry_autotune(fbl_geometry *g, int32_t x_dtype, int32_t n
  * does), 2 the volume staged through shared memory by TMA brick copies (8 columns per
  * block whatever k1_cols; its bounded waits report FBL_E_TIMEOUT from the next
  * synchronous call on the geometry, the results stay correct); k2_vpl = the
- * backprojector's work per warp: 2, 4, 8 or 16 consecutive voxels per lane of
- * one voxel column, or 24 / 28 for a 2x2 group of voxel columns with 4 / 8
- * voxels per lane in each (a detector column's z-profile in a plane is then
- * formed once for its two in-plane neighbours; the sums are the same);
- * FBL_E_INVAL otherwise.  The batched solver runs k1_split 2 volumes with the
- * loads-ahead loop. */
+ * backprojector's work per warp: 2 or 4 (24 the same) = one voxel column, with
+ * that many consecutive voxels per lane; 8, 16 and 28 = strips of 8 voxel
+ * columns, 6 voxels per lane for 16, else 4 or 8, whichever fills nz with less
+ * work (28 and 8 are the same); a new geometry starts with 8 / 1 and a k2_vpl by
+ * its volume's size; FBL_E_INVAL otherwise.  The batched solver runs k1_split 2
+ * volumes with the loads-ahead loop. */
 FBL_API fbl_status geometry_set_launch(fbl_geometry *g, int32_t k1_cols, int32_t k1_split,
                                        int32_t k2_vpl);
 

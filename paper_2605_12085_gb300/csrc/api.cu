@@ -294,7 +294,7 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
     dg.cz_fx = (long long)std::llround(cxyz[2] * FX_ONE);
     dg.k1_cols = 8;
     dg.k1_split = 1;
-    dg.k2_vpl = 4;
+    dg.k2_vpl = backproject_default_config(d.nx, d.ny, d.nz);
     // detector rows with a crossing in (k - 1, k + 1) on one column: at most
     // floor(2 max_inv) + 1
     dg.ntap = (int)std::floor(2.0 * max_inv * 1.0001 + 0.002) + 1;
@@ -1843,7 +1843,8 @@ struct fbl_batch {
     int device = -1;
     int n_vol = 0;
     std::vector<fbl_solver *> sv;   // per-volume state and buffers
-    std::vector<int> order;         // volumes in tile order (largest first)
+    std::vector<int> order;         // volumes in tile order (K2 in strips first, then largest first)
+    int strip_vols = 0;             // volumes whose K2 runs in strips
     int x_dtype = FBL_F32, b_dtype = FBL_F32;
     int cols = 8, split = 1, vpl = 4, ntap = 1;
     // descriptor blob: BatchHdr, BatchVol[n_vol] (tile order), view lists
@@ -1863,7 +1864,7 @@ struct fbl_batch {
 
 namespace {
 
-constexpr int BATCH_SITES = 4;  // persistent launch sites: K1 residual, K2, K3, K1 objective
+constexpr int BATCH_SITES = 5;  // persistent launch sites: K1 residual, K2, K3, K1 objective, K2 in strips
 
 void batch_free(fbl_batch *bt) {
     if (bt->exec) cudaGraphExecDestroy(bt->exec);
@@ -1906,7 +1907,8 @@ fbl_status batch_build_graph(fbl_batch *bt) {
     cudaError_t e = launch_batch_project(PROJ_RESID, hdr, vols, bt->x_dtype, bt->b_dtype, bt->cols,
                                          bt->d_ctr + 0, cs);
     if (e == cudaSuccess) e = launch_batch_reduce(hdr, vols, n, 0, 1, 0, 0, cs);
-    if (e == cudaSuccess) e = launch_batch_backproject(hdr, vols, bt->ntap, bt->d_ctr + 2, cs);
+    if (e == cudaSuccess && bt->strip_vols > 0) e = launch_batch_strips(hdr, vols, bt->d_ctr + 8, cs);
+    if (e == cudaSuccess && bt->strip_vols < n) e = launch_batch_backproject(hdr, vols, bt->ntap, bt->d_ctr + 2, cs);
     if (e == cudaSuccess) e = launch_batch_reduce(hdr, vols, n, 1, 1, 5, 0, cs);
     if (e == cudaSuccess) e = launch_batch_propose(vols, n, bt->have_mlp ? bt->d_mlp : nullptr, bt->margin, cs);
     if (e == cudaSuccess) e = launch_batch_ls_init(blob_hdr(bt, true), vols, n, cs);
@@ -2068,6 +2070,7 @@ fbl_status batch_iterate(fbl_batch *bt, const void *const *b, const char *b_dev,
         cfg.n_theta = d.n_views;
     }
     for (int ph = 0; ph < 3; ++ph) hh->total[ph] = first[ph];
+    hh->strip_tiles = bt->strip_vols < n ? hv[bt->strip_vols].first[1] : first[1];
     auto fail_all = [&](fbl_status r) {
         for (int v = 0; v < n; ++v) restore(v);
         return r;
@@ -2125,7 +2128,7 @@ fbl_status batch_iterate(fbl_batch *bt, const void *const *b, const char *b_dev,
         }
     }
     bt->k += 1;
-    bt->launches += 6 + 5 * (int64_t)max_trials;
+    bt->launches += (bt->strip_vols > 0 && bt->strip_vols < n ? 7 : 6) + 5 * (int64_t)max_trials;
     if (first_bad != FBL_OK) {
         if (first_bad == FBL_E_NONFINITE)
             return fail(FBL_E_NONFINITE, "fblisa_batch_step: volume %d: non-finite objective or reduction", bad_v);
@@ -2192,7 +2195,10 @@ extern "C" fbl_status fblisa_batch_create(const fbl_geometry *const *geoms, cons
     }
     bt->order.resize(n_vol);
     for (int v = 0; v < n_vol; ++v) bt->order[v] = v;
+    for (int v = 0; v < n_vol; ++v) bt->strip_vols += k2_is_strips(geoms[v]->dg.k2_vpl) ? 1 : 0;
     std::stable_sort(bt->order.begin(), bt->order.end(), [&](int a, int c) {
+        const bool sa = k2_is_strips(geoms[a]->dg.k2_vpl), sc = k2_is_strips(geoms[c]->dg.k2_vpl);
+        if (sa != sc) return sa;
         const fbl_geometry_desc &da = geoms[a]->desc, &dc = geoms[c]->desc;
         return (int64_t)da.nx * da.ny * da.nz > (int64_t)dc.nx * dc.ny * dc.nz;
     });

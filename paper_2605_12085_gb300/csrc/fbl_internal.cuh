@@ -129,10 +129,10 @@ struct DevGeom {
     float sod, sdd, inv_du;
     float hwu;                   // half width, in columns, of a voxel's column footprint
     int ntap;                    // detector rows that can touch one voxel in one column
-    // launch configuration (chosen by the autotuner; defaults 8 / 1 / 4)
+    // launch configuration (by the autotuner; defaults 8 / 1 / by the volume's size)
     int k1_cols;                 // projector: detector columns per block (4 or 8)
     int k1_split;                // projector plane loop: 0 plain, 1 loads one sample ahead, 2 TMA-staged bricks
-    int k2_vpl;                  // backprojector: consecutive voxels per lane (2, 4, 8 or 16)
+    int k2_vpl;                  // backprojector: voxel columns (2, 4, 24) or strips (8, 16, 28)
     long long cz_fx;             // cz in Q.40
     const float4 *colA;          // [n_views][nu] (qb0, qb1, zc0, zc1) in FP32, for range estimates
     const FxCol *colF;           // [n_views][nu] exact fixed-point constants
@@ -176,6 +176,32 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
                                int n_sel, float scale, float *gzi, cudaStream_t st,
                                double *g2_partials = nullptr);
 int backproject_num_partials(const DevGeom &g);
+// The k2_vpl a new geometry starts with.
+int backproject_default_config(int nx, int ny, int nz);
+
+struct BpArgs {
+    DevGeom g;
+    const float *rt;
+    const int32_t *views;
+    int n_sel;
+    float scale;
+    float *gzi;
+    double *g2_partials;  // optional: per-block sum of the squared gradient
+};
+// The backprojector in strips (k_strips.cu): blocks of STRIP_EDGE x STRIP_EDGE
+// voxel columns and 32 strip_zp voxels along z.  A span of 32 ZP voxels costs
+// about ZP + 1.2 (8, 6 and 4 voxels per lane measured 0.90, 1.01 and 1.02 ps per
+// voxel and view where nz is a multiple of the span).
+constexpr int STRIP_EDGE = 8;
+__host__ __device__ __forceinline__ bool k2_is_strips(int k2_vpl) { return k2_vpl == 8 || k2_vpl == 16 || k2_vpl == 28; }
+__host__ __device__ __forceinline__ float strip_cost(int nz, int zp) {
+    return (float)((nz + 32 * zp - 1) / (32 * zp)) * ((float)zp + 1.2f);
+}
+__host__ __device__ __forceinline__ int strip_zp(int k2_vpl, int nz) {
+    if (k2_vpl == 16) return 6;
+    return strip_cost(nz, 4) < strip_cost(nz, 8) ? 4 : 8;
+}
+cudaError_t launch_strips(const BpArgs &a, dim3 grid, int zp, cudaStream_t st);
 
 // x_bar = min(max(x - alpha*g - alpha*mu, 0), xmax) on the solver's state:
 // reads vol (current x) and gzi, writes trial; partials[3][nblk] =
@@ -305,6 +331,7 @@ struct BatchVol {
 
 struct BatchHdr {
     int n_vol;
+    int strip_tiles;              // K2 tiles of the volumes that run in strips (first in the tile order)
     int total[3];                 // K1, K2, K3 tiles over all volumes
     int rtotal[2];                // this trial round: K1 / K3 tiles of the searching volumes
 };
@@ -337,6 +364,19 @@ __device__ __forceinline__ void stage_words(void *dst, const void *src, size_t b
     for (int q = tid; q < n; q += nthreads) ((int *)dst)[q] = ((const int *)src)[q];
 }
 
+// The end of a persistent kernel: the last block to leave resets its counter for
+// the next launch.
+__device__ __forceinline__ void batch_leave(int *ctr) {
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        __threadfence();
+        if (atomicAdd(ctr + 1, 1) == (int)gridDim.x - 1) {
+            ctr[0] = 0;
+            ctr[1] = 0;
+            __threadfence();
+        }
+    }
+}
+
 // A volume still inside its line search (neither accepted nor stopped).
 __device__ __forceinline__ bool batch_searching(const LSState &ls) {
     return ls.accepted == 0 && ls.status == 0;
@@ -349,8 +389,10 @@ __device__ __forceinline__ bool batch_searching(const LSState &ls) {
 cudaError_t launch_batch_project(int mode, const BatchHdr *hdr, BatchVol *vols, int x_dtype,
                                  int b_dtype, int cols, int *ctr, cudaStream_t st);
 // Gradient of every volume (scale and views from the descriptor), with the
-// per-tile sums of the squared gradient; each volume keeps its own voxels per
-// lane (g.k2_vpl); ntap >= every volume's g.ntap.
+// per-tile sums of the squared gradient; each volume keeps its own launch
+// configuration (g.k2_vpl): the ones in strips by the first launch, the others by
+// the second (ntap >= every volume's g.ntap).
+cudaError_t launch_batch_strips(const BatchHdr *hdr, BatchVol *vols, int *ctr, cudaStream_t st);
 cudaError_t launch_batch_backproject(const BatchHdr *hdr, BatchVol *vols, int ntap, int *ctr,
                                      cudaStream_t st);
 // Prox + (2.3) sums of the volumes still searching, alpha from their state.

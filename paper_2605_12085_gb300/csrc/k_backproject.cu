@@ -7,11 +7,13 @@
 // y-planes), with weight wb * wz: wb from the in-plane crossing q_b(m) of its
 // detector column, wz from the vertical crossing q_z(m) of its row.
 //
-// Work decomposition.  A warp owns 32*VPL voxels of one (i, j) column along z
-// (lane l holds the VPL consecutive voxels k0 + VPL*l ...; VPL = 2, 4, 8 or
-// 16), or of a 2x2 group of such columns (VPL = 4 or 8), chosen by the
-// autotuner: the kernel is issue bound, and the per-column setup below is
-// paid once per lane for VPL voxels.  Everything that depends only on (i, j)
+// Two forms.  Volumes large enough to fill the GPU run in strips (k_strips.cu).
+// Smaller ones run here, one voxel column per warp: many more and shorter warps
+// (64^3, 10 views: 23.9 against 36 us; 16 volumes of 24^3..80^3 in a batch: 0.82
+// against 0.94 ms per iteration).
+//
+// A warp owns 32*VPL voxels of one (i, j) column along z (lane l holds the VPL
+// consecutive voxels k0 + VPL*l ..; VPL = 2 or 4).  Everything that depends only on (i, j)
 // and the view -- the candidate columns within hwu of the voxel column's
 // projection, each column's family, plane m, exact in-plane weight wb (from
 // the same Q.40 crossing K1 uses) and vertical step -- is uniform over the
@@ -36,26 +38,11 @@ namespace {
 
 constexpr int K2_LANES = 32;
 
-// Launch configuration of the backprojector: k2_vpl in {2, 4, 8, 16} is one
-// voxel column per warp with that many consecutive voxels per lane; 24 and 28
-// are a 2x2 group of voxel columns per warp (k2_tile22) with 4 or 8 voxels per
-// lane in each (the same sums, bit for bit).
-__host__ __device__ __forceinline__ bool k2_group_of(const DevGeom &g) { return g.k2_vpl == 24 || g.k2_vpl == 28; }
-__host__ __device__ __forceinline__ int k2_vpl_of(const DevGeom &g) {
-    if (k2_group_of(g)) return g.k2_vpl - 20;
-    return (g.k2_vpl == 2 || g.k2_vpl == 8 || g.k2_vpl == 16) ? g.k2_vpl : 4;
-}
+// Launch configuration of the backprojector: k2_vpl 2 and 4 (24 the same) are
+// one voxel column per warp with that many consecutive voxels per lane; 8 and 28
+// are strips with 4 or 8 voxels per lane, 16 strips with 6.
+__host__ __device__ __forceinline__ int k2_vpl_of(const DevGeom &g) { return g.k2_vpl == 2 ? 2 : 4; }
 constexpr int K2_WARPS = 8;   // consecutive i per block
-
-struct BpArgs {
-    DevGeom g;
-    const float *rt;
-    const int32_t *views;
-    int n_sel;
-    float scale;
-    float *gzi;
-    double *g2_partials;  // optional: per-block sum of the squared gradient
-};
 
 // Packed FP32x2 arithmetic (sm_100 family): the same IEEE operation on each
 // half, so results equal two scalar operations bit for bit.
@@ -194,159 +181,6 @@ __device__ __forceinline__ void column_profile(float (&acc)[VPL], float wb, cons
         column_cells_c<NTAP, VPL, true>(cc, step, add, rcol, lo, d0 + 1.f, lo_max);
 }
 
-// The first row of one (column, plane) window for the lane's first voxel:
-// lo and d0 = q_z(lo) - kfirst in (-1, -1 + step], exact from the Q.40
-// crossing (an FP32 estimate and one correction), as in k2_tile.
-struct ZWin {
-    int lo;
-    float d0, step, inv;
-};
-__device__ __forceinline__ ZWin z_window(const DevGeom &g, const FxCol *cF, int m, int kfirst) {
-    constexpr float kInv24 = 1.0f / 16777216.0f;  // 2^-24 (Q.40 >> 16)
-    const long long kfirst_fx = (long long)kfirst << FX_BITS;
-    const long long Z = __ldg(&cF->h0) + (long long)m * __ldg(&cF->h1);
-    const long long zoff = g.cz_fx - (long long)(g.nv - 1) * Z;
-    ZWin zw;
-    zw.step = (float)(int)(Z >> 15) * kInv24;
-    zw.inv = __fdividef(1.f, zw.step);
-    const float zoff_f = g.cz - (float)(g.nv - 1) * 0.5f * zw.step;
-    int lo = (int)ceilf(((float)kfirst - zoff_f) * zw.inv - zw.inv);
-    const long long d_fx = 2LL * lo * Z + zoff - kfirst_fx;
-    float d0 = (float)(int)(d_fx >> 16) * kInv24;
-    if (d0 <= -1.f) {
-        ++lo;
-        d0 += zw.step;
-    } else if (d0 - zw.step > -1.f) {
-        --lo;
-        d0 -= zw.step;
-    }
-    zw.lo = lo;
-    zw.d0 = d0;
-    return zw;
-}
-
-// In-plane weight of voxel row bb from the crossing floor b0, fraction fb.
-__device__ __forceinline__ float inplane_weight(int b0, float fb, int bb) {
-    return (b0 == bb) ? 1.f - fb : ((b0 + 1 == bb) ? fb : 0.f);
-}
-
-// One warp's 2x2 group of voxel columns (i0 + x, j0 + y), x, y in {0, 1}: for
-// every view and every candidate detector column, the column's two planes of
-// the group (FAMY: planes j0, j0 + 1, in-plane i0, i0 + 1; else the other
-// way round) each give one z-profile, computed once and added to the two
-// voxel columns of that plane with their in-plane weights.  Every voxel gets
-// exactly the terms of k2_tile, in the same column order and the same
-// arithmetic, so the sums are bit-identical.
-template <int NTAP, int VPL, bool FAMY>
-__device__ __forceinline__ void group_column(float (&acc)[2][2][VPL], const DevGeom &g, const FxCol *cF,
-                                             const float *__restrict__ rcol, int i0, int j0, int kfirst,
-                                             int lo_max) {
-    const int mA = FAMY ? j0 : i0, bA = FAMY ? i0 : j0;
-    const int Na = FAMY ? g.ny : g.nx;
-    // the column constants are read where they are used (an L1 broadcast) rather than kept live
-    long long qb = __ldg(&cF->qb0) + (long long)mA * __ldg(&cF->qb1);
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        if (p) qb += __ldg(&cF->qb1);
-        const int m = mA + p;
-        if (m >= Na) break;
-        const int b0 = fx_floor(qb);
-        const float fb = fx_frac(qb);
-        const float w0 = inplane_weight(b0, fb, bA), w1 = inplane_weight(b0, fb, bA + 1);
-        if (w0 == 0.f && w1 == 0.f) continue;
-        const ZWin zw = z_window(g, cF, m, kfirst);
-        float(&a0)[VPL] = acc[FAMY ? 0 : p][FAMY ? p : 0];
-        float(&a1)[VPL] = acc[FAMY ? 1 : p][FAMY ? p : 1];
-        const int cc = cells_rows(zw.inv);
-        // rows per voxel < ntap / 2 on every column of the geometry
-        const bool inside = zw.lo >= -RT_PAD && zw.lo + (VPL * NTAP + 1) / 2 + 2 <= lo_max;
-        auto add = [&](int q, float Pa, float Pb) {
-            pk_fma(w0, w0, Pa, Pb, a0[q], a0[q + 1], a0[q], a0[q + 1]);
-            pk_fma(w1, w1, Pa, Pb, a1[q], a1[q + 1], a1[q], a1[q + 1]);
-        };
-        if (__all_sync(0xffffffffu, inside))
-            column_cells_c<NTAP, VPL, false>(cc, zw.step, add, rcol, zw.lo, zw.d0 + 1.f, lo_max);
-        else
-            column_cells_c<NTAP, VPL, true>(cc, zw.step, add, rcol, zw.lo, zw.d0 + 1.f, lo_max);
-    }
-}
-
-// One block of 8 warps = 4 x 2 groups: voxel columns i in [8 gx, 8 gx + 8),
-// j in [4 gy, 4 gy + 4), z-span bz; the block's sum of squared gradient values
-// goes to *g2_partial (if not NULL).  Called by every thread.
-template <int NTAP, int VPL>
-__device__ __forceinline__ void k2_tile22(const BpArgs &a, int gx, int gy, int bz, double *g2_partial) {
-    const DevGeom &g = a.g;
-    const int lane = threadIdx.x, w = threadIdx.y;
-    const int i0 = 8 * gx + 2 * (w & 3), j0 = 4 * gy + 2 * (w >> 2);
-    const int kfirst = bz * K2_LANES * VPL + VPL * lane;
-    float acc[2][2][VPL];
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y)
-#pragma unroll
-            for (int q = 0; q < VPL; ++q) acc[x][y][q] = 0.f;
-    const int rp = rt_pitch(g.nv);
-    const int nsel = (i0 < g.nx && j0 < g.ny) ? a.n_sel : 0;
-    const int lo_max = g.nv + RT_PAD - NTAP;
-    for (int s = 0; s < nsel; ++s) {
-        const int v = a.views[s];
-        const float2 cs = g.trig[v];
-        // the union of the four voxel columns' candidate windows (k2_tile's),
-        // from the extreme projections (ceil and floor are monotone)
-        float umin = 3.0e38f, umax = -3.0e38f;
-#pragma unroll
-        for (int x = 0; x < 2; ++x)
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                const float xc = ((float)(i0 + x) - g.cx) * g.vx;
-                const float yc = ((float)(j0 + y) - g.cy) * g.vy;
-                const float xi = xc * cs.x + yc * cs.y;
-                const float eta = -xc * cs.y + yc * cs.x;
-                const float iuc = eta * __fdividef(g.sdd, g.sod - xi) * g.inv_du + g.cu;
-                umin = fminf(umin, iuc);
-                umax = fmaxf(umax, iuc);
-            }
-        const int iu_lo = max(0, (int)ceilf(umin - g.hwu));
-        const int iu_hi = min(g.nu - 1, (int)floorf(umax + g.hwu));
-        for (int iu = iu_lo; iu <= iu_hi; ++iu) {
-            const size_t col = (size_t)v * g.nu + iu;
-            const FxCol *cF = g.colF + col;
-            const float *rcol = a.rt + ((size_t)s * g.nu + iu) * rp + RT_PAD;
-            if (g.colB[col].z != 0.f)
-                group_column<NTAP, VPL, true>(acc, g, cF, rcol, i0, j0, kfirst, lo_max);
-            else
-                group_column<NTAP, VPL, false>(acc, g, cF, rcol, i0, j0, kfirst, lo_max);
-        }
-    }
-    float g2 = 0.f;
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y) {
-            const int i = i0 + x, j = j0 + y;
-            if (i < g.nx && j < g.ny) {
-                float *out = a.gzi + ((size_t)j * g.nx + i) * g.nz;
-#pragma unroll
-                for (int q = 0; q < VPL; ++q) {
-                    const int k = kfirst + q;
-                    if (k < g.nz) {
-                        const float val = a.scale * acc[x][y][q];
-                        out[k] = val;
-                        g2 = fmaf(val, val, g2);
-                    }
-                }
-            }
-        }
-    if (g2_partial) {
-        float vv[1] = {g2};
-        double o[1];
-        block_sum_f64<K2_LANES * K2_WARPS, 1>(vv, o);
-        if (threadIdx.x == 0 && threadIdx.y == 0) *g2_partial = o[0];
-    }
-}
-
 // One block's work: voxel columns i = bx*8 .. bx*8+7 of row j, z-span bz;
 // the block's sum of squared gradient values goes to *g2_partial (if not NULL).
 // Called by every thread.
@@ -440,29 +274,19 @@ __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) k2_backproject(const Bp
     k2_tile<NTAP, K2_VPL>(a, blockIdx.x, blockIdx.y, blockIdx.z, a.g2_partials ? a.g2_partials + blk : nullptr);
 }
 
-// At most 80 registers (3 blocks per SM), no spills: 8.55 against 9.22 ms per
-// 40-view launch at 512^3 (8 voxels per lane), and 166.9 against 175.2 ms for
-// all 720 views, with 64 registers, 4 blocks per SM and a few spilled values.
-template <int NTAP, int VPL>
-__global__ void __launch_bounds__(K2_LANES *K2_WARPS, 3) k2_backproject22(const BpArgs a) {
-    const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    k2_tile22<NTAP, VPL>(a, blockIdx.x, blockIdx.y, blockIdx.z, a.g2_partials ? a.g2_partials + blk : nullptr);
-}
-
-// Persistent batched backprojector: the blocks of k2_backproject (or of the
-// 2x2 group kernel) of every volume, taken from an atomic counter.  Each volume
-// keeps its own launch configuration (its geometry's k2_vpl, a warp-uniform
-// switch).  Registers are capped at 64 (4 blocks per SM), what the group tiles
-// need.
+// Persistent batched backprojector: the blocks of k2_backproject of every volume
+// that does not run in strips (the tiles from hdr->strip_tiles on), taken from an
+// atomic counter.  Each volume keeps its own voxels per lane (its geometry's
+// k2_vpl, a warp-uniform switch).
 template <int NTAP>
-__global__ void __launch_bounds__(K2_LANES *K2_WARPS, 4) kb_backproject(const BatchHdr *hdr,
+__global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) kb_backproject(const BatchHdr *hdr,
                                                                         const BatchVol *vols, int *ctr) {
     __shared__ int s_tile;
     __shared__ BpArgs sa;
     const int tid = threadIdx.x + K2_LANES * threadIdx.y;
     const int total = hdr->total[1];
     for (;;) {
-        if (tid == 0) s_tile = atomicAdd(ctr, 1);
+        if (tid == 0) s_tile = hdr->strip_tiles + atomicAdd(ctr, 1);
         __syncthreads();
         const int t = s_tile;
         __syncthreads();
@@ -482,47 +306,27 @@ __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 4) kb_backproject(const Ba
         __syncthreads();
         const BpArgs &a = sa;
         const int local = t - bv.first[1];
-        const int vpl = k2_vpl_of(bv.g);
-        double *gpart = bv.partials + local;
-        if (k2_group_of(bv.g)) {
-            const int gxn = (bv.g.nx + 7) / 8, gyn = (bv.g.ny + 3) / 4;
-            const int gx = local % gxn;
-            const int rest = local / gxn;
-            if (vpl == 8) k2_tile22<NTAP, 8>(a, gx, rest % gyn, rest / gyn, gpart);
-            else k2_tile22<NTAP, 4>(a, gx, rest % gyn, rest / gyn, gpart);
-            continue;
-        }
         const int gx = (bv.g.nx + K2_WARPS - 1) / K2_WARPS;
         const int bx = local % gx;
         const int rest = local / gx;
         const int j = rest % bv.g.ny;
         const int bz = rest / bv.g.ny;
         double *part = bv.partials + local;
-        switch (vpl) {
-            case 2: k2_tile<NTAP, 2>(a, bx, j, bz, part); break;
-            case 8: k2_tile<NTAP, 8>(a, bx, j, bz, part); break;
-            case 16: k2_tile<NTAP, 16>(a, bx, j, bz, part); break;
-            default: k2_tile<NTAP, 4>(a, bx, j, bz, part); break;
-        }
+        if (k2_vpl_of(bv.g) == 2) k2_tile<NTAP, 2>(a, bx, j, bz, part);
+        else k2_tile<NTAP, 4>(a, bx, j, bz, part);
     }
-    if (tid == 0) {
-        __threadfence();
-        if (atomicAdd(ctr + 1, 1) == (int)gridDim.x - 1) {
-            ctr[0] = 0;
-            ctr[1] = 0;
-            __threadfence();
-        }
-    }
+    batch_leave(ctr);
 }
 
 }  // namespace
 
-
 static dim3 k2_grid(const DevGeom &g) {
+    if (k2_is_strips(g.k2_vpl)) {
+        const unsigned span = 32 * strip_zp(g.k2_vpl, g.nz);
+        return dim3((g.nx + STRIP_EDGE - 1) / STRIP_EDGE, (g.ny + STRIP_EDGE - 1) / STRIP_EDGE, (g.nz + span - 1) / span);
+    }
     const int vpl = k2_vpl_of(g);
-    const unsigned gz = (g.nz + K2_LANES * vpl - 1) / (K2_LANES * vpl);
-    if (k2_group_of(g)) return dim3((g.nx + 7) / 8, (g.ny + 3) / 4, gz);
-    return dim3((g.nx + K2_WARPS - 1) / K2_WARPS, g.ny, gz);
+    return dim3((g.nx + K2_WARPS - 1) / K2_WARPS, g.ny, (g.nz + K2_LANES * vpl - 1) / (K2_LANES * vpl));
 }
 
 int backproject_num_partials(const DevGeom &g) {
@@ -530,19 +334,19 @@ int backproject_num_partials(const DevGeom &g) {
     return (int)(gr.x * gr.y * gr.z);
 }
 
+int backproject_default_config(int nx, int ny, int nz) {
+    // fewer than 100 patches of 8 x 8 x 128 (80^3) leave SMs idle: one voxel column
+    // per warp, 64 voxels high where that is enough (64^3, 10 views: 23.9 us with 2
+    // voxels per lane, 28.0 with 4, 36 in strips; 96^3: 48.5 with 4, 37 in strips)
+    const int64_t patches = (int64_t)((nx + 7) / 8) * ((ny + 7) / 8) * ((nz + 127) / 128);
+    if (patches <= 100) return nz <= 64 ? 2 : 4;
+    return strip_cost(nz, 6) < strip_cost(nz, strip_zp(28, nz)) ? 16 : 28;
+}
+
 template <int NT>
 static void launch_k2(int vpl, dim3 grid, dim3 block, cudaStream_t st, const BpArgs &a) {
-    if (k2_group_of(a.g)) {
-        if (vpl == 8) k2_backproject22<NT, 8><<<grid, block, 0, st>>>(a);
-        else k2_backproject22<NT, 4><<<grid, block, 0, st>>>(a);
-        return;
-    }
-    switch (vpl) {
-        case 2: k2_backproject<NT, 2><<<grid, block, 0, st>>>(a); break;
-        case 8: k2_backproject<NT, 8><<<grid, block, 0, st>>>(a); break;
-        case 16: k2_backproject<NT, 16><<<grid, block, 0, st>>>(a); break;
-        default: k2_backproject<NT, 4><<<grid, block, 0, st>>>(a); break;
-    }
+    if (vpl == 2) k2_backproject<NT, 2><<<grid, block, 0, st>>>(a);
+    else k2_backproject<NT, 4><<<grid, block, 0, st>>>(a);
 }
 
 template <class K>
@@ -588,8 +392,9 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
     a.scale = scale;
     a.gzi = gzi;
     dim3 block(K2_LANES, K2_WARPS);
-    const int vpl = k2_vpl_of(g);
     const dim3 grid = k2_grid(g);
+    if (k2_is_strips(g.k2_vpl)) return launch_strips(a, grid, strip_zp(g.k2_vpl, g.nz), st);
+    const int vpl = k2_vpl_of(g);
     switch (g.ntap) {  // rows per voxel and column, fixed per geometry (<= RT_PAD)
         case 1: launch_k2<1>(vpl, grid, block, st, a); break;
         case 2: launch_k2<2>(vpl, grid, block, st, a); break;
