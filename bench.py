@@ -650,8 +650,11 @@ def make_data(fbl, wl, device):
 
 
 def step_units(st, g):
+    """Work an iteration completes: the residual projection, the accepted trial's
+    objective and the backprojection.  A rejected trial's projection ends once its
+    partial sum settles the test (2.3), and is not counted."""
     N_t = st["N_t"]
-    n_proj = st["backtracks"] + 2
+    n_proj = 2
     samples = n_proj * N_t * g.nu * g.nv * g.nx
     voxel_views = N_t * g.nx * g.ny * g.nz
     return samples + voxel_views
@@ -889,8 +892,8 @@ def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
     40-view mini-batches: GUPS over the work an iteration does (every forward
     projection N_t nu nv N samples, the backprojection N_t N^3 voxel-views),
     per-kernel CUDA-event times recorded by the library on the launching
-    stream, and the rooflines of the trial-objective projection (K1), the
-    gradient backprojection (K2) and the prox (K3)."""
+    stream, and the rooflines of the residual projection (K1; a trial's objective
+    may end early), the gradient backprojection (K2) and the prox (K3)."""
     import numpy as np
     import torch
     params = fbl.params_default(alpha0=1e-3, beta=0.5, mu=wl.mu, N0=wl.N0, seed=wl.seed_batches,
@@ -918,7 +921,7 @@ def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
     units = sum(step_units(st, g) for st in stats)
     samples = float(np.mean([active_samples(g, vs) for vs in batches[:3]]))
     N_t = stats[0]["N_t"]
-    k1_ms, k1_n = prof["objective_projection"]
+    k1_ms, k1_n = prof["residual_projection"]
     k2_ms, k2_n = prof["gradient_backprojection"]
     k3_ms, k3_n = prof["prox_reduce"]
     k3_avg = k3_ms / max(k3_n, 1)
@@ -929,7 +932,7 @@ def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
         "gups": units / (ms * 1e-3) / 1e9, "ms_per_iteration": ms / steps, "steps": steps, "warmup": warmup,
         "backtracks_per_iteration": statistics.mean(st["backtracks"] for st in stats),
         "in_volume_samples_per_projection": samples,
-        "roofline_k1": alu_roofline("k1_project, trial objective (Step 2c, eq. (2.3))", K1_OPS_PER_SAMPLE,
+        "roofline_k1": alu_roofline("k1_project, residual (Step 2b, eq. (2.5))", K1_OPS_PER_SAMPLE,
                                     samples, k1_ms / max(k1_n, 1), g.n_vox * 4 + N_t * g.nu * g.nv * 4, clk,
                                     peaks),
         "roofline_k2": alu_roofline("k2_backproject, gradient (Step 2b, eq. (2.5))", K2_OPS_PER_SAMPLE,

@@ -1088,10 +1088,14 @@ fbl_status build_graph(fbl_solver *s, fbl_solver::GraphEntry &ge) {
         e = cudaStreamBeginCaptureToGraph(cb, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             cudaError_t eb = launch_prox_zi_dev(ge.st, s->L, s->grad, s->d_ls, ge.tr, xdt, s->partials, &npp, cb);
-            if (eb == cudaSuccess) eb = launch_reduce(s->partials, npp, npp, 3, s->d_sc + 1, cb);
+            double *stop = project_may_stop(s->dg, N) ? s->d_sc + 6 : nullptr;
+            if (eb == cudaSuccess)
+                eb = stop ? launch_reduce_trial(s->partials, npp, s->d_sc, s->d_ls, 0.0, 0.0, 0,
+                                                std::max(s->dg.vx, s->dg.vy), cb)
+                          : launch_reduce(s->partials, npp, npp, 3, s->d_sc + 1, cb);
             if (eb == cudaSuccess)
                 eb = launch_project(PROJ_NORM, s->dg, ge.tr, s->L, xdt, s->d_views, N, ge.bd, s->p.b_dtype,
-                                    ge.bmap, nullptr, FBL_F32, s->partials, &np2, cb);
+                                    ge.bmap, nullptr, FBL_F32, s->partials, &np2, cb, stop);
             if (eb == cudaSuccess) eb = launch_reduce(s->partials, np2, np2, 1, s->d_sc + 4, cb);
             if (eb == cudaSuccess) eb = launch_ls_decide(s->d_ls, s->d_ps, s->d_sc, cond, cb);
             cudaError_t ee = cudaStreamEndCapture(cb, &body);
@@ -1349,14 +1353,19 @@ fbl_status solver_iterate(fbl_solver *s, const void *b, bool b_dev, fbl_step_sta
     bool accepted = false;
     int bt = 0;
     double rho0 = 0, rho1 = 0, gTd = 0, dd = 0, f_x = 0, f_xb = 0, rhs = 0;
+    double *stop = project_may_stop(s->dg, N) ? s->d_sc + 6 : nullptr;
     for (bt = 0; bt <= s->p.max_backtracks; ++bt) {
         int npp = 0;
         CK(prof_launch(s, 3, st, [&] { return solver_prox(s, alpha, &npp, st); }), "prox kernel");
-        CK(prof_launch(s, 4, st, [&] { return launch_reduce(s->partials, npp, npp, 3, s->d_sc + 1, st); }),
+        CK(prof_launch(s, 4, st, [&] {
+               return stop ? launch_reduce_trial(s->partials, npp, s->d_sc, s->d_ls, alpha, scale,
+                                                 bt == s->p.max_backtracks, std::max(s->dg.vx, s->dg.vy), st)
+                           : launch_reduce(s->partials, npp, npp, 3, s->d_sc + 1, st);
+           }),
            "reduce");
         CK(prof_launch(s, 1, st, [&] {
                return launch_project(PROJ_NORM, s->dg, s->tr, s->L, xdt, s->d_views, N,
-                                     bd, s->p.b_dtype, bmap, nullptr, FBL_F32, s->partials, &np, st);
+                                     bd, s->p.b_dtype, bmap, nullptr, FBL_F32, s->partials, &np, st, stop);
            }),
            "objective kernel");
         CK(prof_launch(s, 4, st, [&] { return launch_reduce(s->partials, np, np, 1, s->d_sc + 4, st); }),

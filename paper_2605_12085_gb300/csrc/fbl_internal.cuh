@@ -156,14 +156,21 @@ cudaError_t launch_zi_to_natural(const float *gzi, float *x, int nx, int ny, int
 // mode STORE: out[s][iv][iu] = A_{views[s]} x  (out_dtype)
 // mode RESID: out = rt[s][iu][RT_PAD + iv] = W * (A x - b) as float32, partials += r^2
 // mode NORM:  partials += (A x - b)^2 only
+// stop (mode NORM): two doubles, a running sum of the finished blocks' partials
+// and a limit (launch_reduce_trial); once the sum is above the limit the blocks
+// that have not started write a partial of 0 and leave.
 // b_views: device list mapping slot s to the view index inside b (NULL: b is
 // already the batch, slot s at index s).  b is [view][nv][nu].
 cudaError_t launch_project(int mode, const DevGeom &g, const void *vol, ZLayout L, int x_dtype,
                            const int32_t *views,
                            int n_sel, const void *b, int b_dtype, const int32_t *b_views,
                            void *out, int out_dtype, double *partials, int *n_partials,
-                           cudaStream_t st);
+                           cudaStream_t st, double *stop = nullptr);
 int project_num_partials(const DevGeom &g, int n_sel);
+// Whether a trial objective over n_sel views has blocks that could leave early:
+// more than one wave of them.  (Within one wave the limit would only cost: 64^3, 10
+// views, 2 us a trial.)
+bool project_may_stop(const DevGeom &g, int n_sel);
 
 // rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu] (the row weight folded in for K2);
 // the pad entries are left untouched (the caller zeroes them once).
@@ -268,6 +275,7 @@ struct LSState {
     int trials, max_backtracks, accepted, status, force_reject;
     int j_start;                // first trial = alpha0 * beta^j_start
     int N_t, n_theta;
+    int ticket;                 // blocks of the trial's reduction that are done (0 between launches)
     float pred;                 // network output (backtracks predicted)
     float feat[MLP_IN];         // the proposal's input features
 };
@@ -285,6 +293,13 @@ struct PropState {
 cudaError_t launch_propose(LSState *ls, const PropState *ps, const double *sc, const float *params,
                            float margin, cudaStream_t st);
 cudaError_t launch_ls_init(LSState *ls, cudaStream_t st);
+// Trial sums of the prox (sc[1..3] = gTd, dd, l1 from partials[3][n]), and the
+// limit the trial's rho1 has to stay below: sc[6] = 0 (running sum), sc[7] = the
+// rho1 above which (2.3) is certain to fail, +inf where the trial's objective has
+// to be complete.  The step and the trial count are ls's, or alpha and last
+// (1: no further trial) where alpha > 0.  wmax: a bound of the geometry's voxel sizes.
+cudaError_t launch_reduce_trial(const double *partials, int n, double *sc, LSState *ls, double alpha, double scale,
+                                int last, float wmax, cudaStream_t st);
 // Evaluate (2.3) on sc = [rho0, gTd, dd, l1, rho1]; accept (and record the
 // iteration in ps), or shrink the step and request another trial (the WHILE
 // condition), or stop with a status.
@@ -318,7 +333,7 @@ struct BatchVol {
     float *rt;                    // weighted residual rt[s][iu][RT_PAD + iv]
     float *grad;                  // gradient [j][i][k]
     double *partials;             // per-tile partial sums
-    double *sc;                   // [8] scalars (rho0, gTd, dd, l1, rho1, g2)
+    double *sc;                   // [8] scalars (rho0, gTd, dd, l1, rho1, g2, running rho1, its limit)
     LSState *ls;                  // line-search state
     PropState *ps;                // proposal statistics (persistent)
     float scale;                  // n_theta / N_t

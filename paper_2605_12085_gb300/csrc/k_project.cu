@@ -56,7 +56,17 @@ struct ProjArgs {
     const int32_t *b_views;
     void *out;
     double *partials;
+    double *stop;  // NORM: running sum of the blocks' partials and its limit, or NULL
+    int first;     // blocks of the first wave (they need not look at stop)
 };
+
+// The order a trial objective takes its bands of detector rows in: the middle
+// first, where the rays meet most of the volume, so that the running sum of a
+// trial that will be rejected passes its limit early.
+__device__ __forceinline__ int centre_out(int z, int n) {
+    const int mid = (n - 1) / 2;
+    return (z & 1) ? mid + (z + 1) / 2 : mid - z / 2;
+}
 
 // Intersect [mlo, mhi] with the real interval where lo < c0 + m*c1 < hi.
 __device__ __forceinline__ void clip_affine(float c0, float c1, float lo, float hi, float &mlo,
@@ -329,7 +339,10 @@ __device__ __forceinline__ void k1_tile(const ProjArgs &a, int cb, int s, int ba
         float vv[1] = {r2};
         double out[1];
         block_sum_f64<32 * COLS, 1>(vv, out);
-        if (threadIdx.x == 0 && threadIdx.y == 0) *partial = out[0];
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
+            *partial = out[0];
+            if (MODE == PROJ_NORM && a.stop) atomicAdd(a.stop, out[0]);
+        }
     }
 }
 
@@ -339,8 +352,24 @@ __device__ __forceinline__ void k1_tile(const ProjArgs &a, int cb, int s, int ba
 // a 32-register cap is slower).
 template <typename TX, typename TB, typename TO, int MODE, int COLS, bool PIPE>
 __global__ void __launch_bounds__(32 * COLS, 48 / COLS) k1_project(const ProjArgs a) {
-    const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    k1_tile<TX, TB, TO, MODE, COLS, PIPE>(a, blockIdx.x, blockIdx.y, blockIdx.z,
+    const int band = MODE == PROJ_NORM ? centre_out(blockIdx.z, gridDim.z) : blockIdx.z;
+    const size_t blk = ((size_t)band * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    if (MODE == PROJ_NORM && a.stop) {
+        // a trial whose sum has passed the limit is rejected whatever the rest of it
+        // is: the blocks still to come leave
+        const size_t at = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        if (at >= a.first) {
+            __shared__ int s_done;
+            const bool lead = threadIdx.x == 0 && threadIdx.y == 0;
+            if (lead) s_done = __ldcg(a.stop) > __ldcg(a.stop + 1);
+            __syncthreads();
+            if (s_done) {
+                if (lead) a.partials[blk] = 0.0;
+                return;
+            }
+        }
+    }
+    k1_tile<TX, TB, TO, MODE, COLS, PIPE>(a, blockIdx.x, blockIdx.y, band,
                                            MODE != PROJ_STORE ? a.partials + blk : nullptr);
 }
 
@@ -655,7 +684,7 @@ __global__ void __launch_bounds__(32 * TMA_COLS) k1_project_tma(const ProjArgs a
 template <typename TX, typename TB, int MODE, int COLS>
 __global__ void __launch_bounds__(32 * COLS, 48 / COLS) kb_project(const BatchHdr *hdr, const BatchVol *vols,
                                                                    int *ctr) {
-    __shared__ int s_tile;
+    __shared__ int s_tile, s_done;
     __shared__ ProjArgs sa;
     const int tid = threadIdx.x + 32 * threadIdx.y;
     // the trial objective covers only the volumes still searching in this trial
@@ -678,15 +707,25 @@ __global__ void __launch_bounds__(32 * COLS, 48 / COLS) kb_project(const BatchHd
             sa.b_views = bv.b_views;
             sa.out = bv.rt;
             sa.partials = bv.partials;
+            sa.stop = MODE == PROJ_NORM ? bv.sc + 6 : nullptr;
+            if (MODE == PROJ_NORM) s_done = __ldcg(bv.sc + 6) > __ldcg(bv.sc + 7);
         }
         __syncthreads();
         const ProjArgs &a = sa;
-        const int local = t - (MODE == PROJ_NORM ? bv.rfirst[0] : bv.first[0]);
+        int local = t - (MODE == PROJ_NORM ? bv.rfirst[0] : bv.first[0]);
         const int ncb = (bv.g.nu + COLS - 1) / COLS;
         const int cb = local % ncb;
         const int rest = local / ncb;
         const int s = rest % bv.N_t;
-        const int band = rest / bv.N_t;
+        int band = rest / bv.N_t;
+        if (MODE == PROJ_NORM) {  // as in k1_project
+            band = centre_out(band, (bv.g.nv + K1_ROWS - 1) / K1_ROWS);
+            local = (band * bv.N_t + s) * ncb + cb;
+            if (s_done) {
+                if (tid == 0) bv.partials[local] = 0.0;
+                continue;
+            }
+        }
         if (bv.g.k1_split)  // each volume keeps its own plane-loop form
             k1_tile<TX, TB, float, MODE, COLS, true>(a, cb, s, band, bv.partials + local);
         else
@@ -824,10 +863,24 @@ int project_num_partials(const DevGeom &g, int n_sel) {
     return ((g.nu + cols - 1) / cols) * n_sel * ((g.nv + K1_ROWS - 1) / K1_ROWS);
 }
 
+// Blocks of k1_project that are resident at once.
+static int first_wave(const DevGeom &g) {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
+    }();
+    return sms * (48 / (g.k1_cols == 4 ? 4 : 8));
+}
+
+bool project_may_stop(const DevGeom &g, int n_sel) {
+    return g.k1_split != 2 && project_num_partials(g, n_sel) > first_wave(g);
+}
+
 cudaError_t launch_project(int mode, const DevGeom &g, const void *vol, ZLayout L, int x_dtype,
                            const int32_t *views, int n_sel, const void *b, int b_dtype,
                            const int32_t *b_views, void *out, int out_dtype, double *partials,
-                           int *n_partials, cudaStream_t st) {
+                           int *n_partials, cudaStream_t st, double *stop) {
     if (n_sel <= 0) {
         if (n_partials) *n_partials = 0;
         return cudaSuccess;
@@ -841,6 +894,8 @@ cudaError_t launch_project(int mode, const DevGeom &g, const void *vol, ZLayout 
     a.b_views = b_views;
     a.out = out;
     a.partials = partials;
+    a.stop = stop;
+    a.first = first_wave(g);
     if (n_partials) *n_partials = project_num_partials(g, n_sel);
     switch (x_dtype) {
         case FBL_BF16: return launch_bdt<__nv_bfloat16>(mode, b_dtype, out_dtype, a, n_sel, st);

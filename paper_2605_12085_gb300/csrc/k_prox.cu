@@ -213,8 +213,40 @@ __global__ void __launch_bounds__(R_NT) k_reduce(const double *__restrict__ part
     if (threadIdx.x == 0) out[c] = s;
 }
 
+// The limit of a trial's rho1 (see launch_reduce_trial).  The trial is rejected
+// when f_N(x_bar) > rhs, and f_N(x_bar) is a sum of squares: a partial sum above
+// the limit settles it.  The margin of 1e-9 covers the order of the FP64 sums
+// (at most 2^20 terms).  The objective is completed where a rejected trial's
+// value is reported or checked: at the last trial, and where a square could
+// overflow FP32 (the bounds keep |A x_bar - b| below 1e18, so a trial that is
+// stopped early cannot hide a non-finite objective).
+__device__ __forceinline__ void trial_limit(double *sc, double alpha, double scale, bool last, float wmax) {
+    const double rho0 = __ldcg(sc), gTd = __ldcg(sc + 1), dd = __ldcg(sc + 2), l1 = __ldcg(sc + 3);
+    const double half = 0.5 * scale, rhs = half * rho0 + gTd + dd / (2.0 * alpha);
+    const bool bounded = rho0 < 1e24 && dd < 1e20 && l1 < 1e15 && wmax < 100.f && isfinite(rhs);
+    sc[6] = 0.0;
+    sc[7] = bounded && !last ? fmax(rhs, 0.0) / half * (1.0 + 1e-9) : INFINITY;
+}
+
+// k_reduce of the three sums of a trial; the last of its three blocks sets the
+// trial's limit.
+__global__ void __launch_bounds__(R_NT) k_reduce_trial(const double *__restrict__ partials, int n, double *sc,
+                                                       LSState *ls, double alpha, double scale, int last, float wmax) {
+    const int c = blockIdx.x;
+    const double s = block_reduce_fixed(partials + (size_t)c * n, n);
+    if (threadIdx.x != 0) return;
+    sc[1 + c] = s;
+    __threadfence();
+    if (atomicAdd(&ls->ticket, 1) != 2) return;
+    ls->ticket = 0;
+    __threadfence();
+    if (alpha > 0.0) trial_limit(sc, alpha, scale, last != 0, wmax);
+    else trial_limit(sc, ls->alpha, ls->scale, ls->trials >= ls->max_backtracks, wmax);
+}
+
 // One block per (volume, component): the same fixed order as k_reduce over the
-// volume's tiles of phase ph (stride = its tile count).
+// volume's tiles of phase ph (stride = its tile count).  The three sums of a trial
+// (ph 2) end with the trial's limit, as k_reduce_trial.
 __global__ void __launch_bounds__(R_NT) kb_reduce(const BatchVol *vols, int ph, int ncomp, int slot,
                                                   int searching_only) {
     const int v = blockIdx.x / ncomp, c = blockIdx.x % ncomp;
@@ -222,7 +254,15 @@ __global__ void __launch_bounds__(R_NT) kb_reduce(const BatchVol *vols, int ph, 
     if (searching_only && !batch_searching(*bv.ls)) return;  // block-uniform
     const int n = bv.tiles[ph];
     const double s = block_reduce_fixed(bv.partials + (size_t)c * n, n);
-    if (threadIdx.x == 0) bv.sc[slot + c] = s;
+    if (threadIdx.x != 0) return;
+    bv.sc[slot + c] = s;
+    if (ph != 2) return;
+    LSState &ls = *bv.ls;
+    __threadfence();
+    if (atomicAdd(&ls.ticket, 1) != 2) return;
+    ls.ticket = 0;
+    __threadfence();
+    trial_limit(bv.sc, ls.alpha, ls.scale, ls.trials >= ls.max_backtracks, fmaxf(bv.g.vx, bv.g.vy));
 }
 
 }  // namespace
@@ -353,6 +393,12 @@ cudaError_t launch_batch_reduce(const BatchHdr *hdr, BatchVol *vols, int n_vol, 
                                 int slot, int searching_only, cudaStream_t st) {
     (void)hdr;
     kb_reduce<<<n_vol * ncomp, R_NT, 0, st>>>(vols, ph, ncomp, slot, searching_only);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_trial(const double *partials, int n, double *sc, LSState *ls, double alpha, double scale,
+                                int last, float wmax, cudaStream_t st) {
+    k_reduce_trial<<<3, R_NT, 0, st>>>(partials, n, sc, ls, alpha, scale, last, wmax);
     return cudaGetLastError();
 }
 
