@@ -807,13 +807,11 @@ extern "C" fbl_status prox_tv(const int32_t dims[3], const float *v, double lamb
     const void *vd = nullptr;
     fbl_status st;
     if ((st = device_input(v, n * sizeof(float), vs, &vd, s))) return st;
-    // two dual pairs: (caller's device q or scratch, r0), (q1, r1); and y
+    // three dual buffers, the first the caller's where it is on the device
     const bool q_dev = q && is_device_ptr(q);
-    CK(scratch.alloc((q_dev ? 10 : 13) * n * sizeof(float), s), "scratch");
+    CK(scratch.alloc((q_dev ? 6 : 9) * n * sizeof(float), s), "scratch");
     float *base = (float *)scratch.p;
-    float *const qp[2] = {q_dev ? q : base + 10 * n, base + 3 * n};
-    float *const rp[2] = {base, base + 6 * n};
-    float *y = base + 9 * n;
+    float *const qp[3] = {q_dev ? q : base + 6 * n, base, base + 3 * n};
     const float *q_start = nullptr;
     if (q_in) {
         if (!q_dev) CK(cudaMemcpyAsync(qp[0], q, 3 * n * sizeof(float), cudaMemcpyHostToDevice, s), "q H2D");
@@ -825,9 +823,10 @@ extern "C" fbl_status prox_tv(const int32_t dims[3], const float *v, double lamb
         CK(xs.alloc(n * sizeof(float), s), "output staging");
         xd = (float *)xs.p;
     }
-    int cur = 1;  // the start goes to pair 1 (it reads pair 0's q)
-    CK(launch_tv_prox((const float *)vd, nx, ny, nz, (float)lambda, (float)x_max, iters, q_start, qp, rp, y, xd,
-                      &cur, s),
+    // the start's buffer, such that the last dual, `iters` places on, is in the
+    // caller's (a start that is read from there goes to another one)
+    int cur = q_start && iters % 3 == 0 ? 1 : (3 - iters % 3) % 3;
+    CK(launch_tv_prox((const float *)vd, nx, ny, nz, (float)lambda, (float)x_max, iters, q_start, qp, xd, &cur, s),
        "TV prox kernels");
     if (q) {
         if (q_dev && cur != 0)
@@ -915,9 +914,9 @@ struct fbl_solver {
     PropState *h_ps = nullptr;                    // pinned mirror (host-loop mode)
     float *d_mlp = nullptr;                       // network parameters, NULL until set
     float margin = 0.25f;
-    // TV prox (reg = FBL_REG_TV): b, y, then (q[3], r[3]) twice, consecutive FP32 volumes
+    // TV prox (reg = FBL_REG_TV): b, then three duals of 3 volumes, consecutive FP32
     float *tv_buf = nullptr;
-    int tv_cur = 0;                               // the pair holding the previous prox's dual
+    int tv_cur = 0;                               // the buffer holding the previous prox's dual
     bool tv_have_q = false;
 };
 
@@ -932,11 +931,11 @@ cudaError_t solver_prox(fbl_solver *s, double alpha, int *npp, cudaStream_t st) 
         return launch_prox_zi(s->st, s->L, s->grad, (float)alpha, (float)(alpha * s->p.mu), (float)s->p.x_max,
                               s->tr, xdt, s->partials, npp, st);
     const size_t n = (size_t)s->L.nx * s->L.ny * s->L.nz;
-    float *b = s->tv_buf, *y = b + n;
-    float *const q[2] = {y + n, y + 7 * n}, *const r[2] = {y + 4 * n, y + 10 * n};
+    float *b = s->tv_buf;
+    float *const q[3] = {b + n, b + 4 * n, b + 7 * n};
     const int warm = s->p.tv_warm && s->tv_have_q;
     cudaError_t e = launch_tv_prox_zi(s->st, s->L, s->grad, (float)alpha, (float)(alpha * s->p.mu),
-                                      (float)s->p.x_max, s->p.tv_iters, warm, b, q, r, &s->tv_cur, y, s->tr, xdt,
+                                      (float)s->p.x_max, s->p.tv_iters, warm, b, q, &s->tv_cur, s->tr, xdt,
                                       s->partials, npp, st);
     if (e == cudaSuccess) s->tv_have_q = true;
     return e;
@@ -1707,8 +1706,8 @@ extern "C" fbl_status fblisa_create(const fbl_geometry *g, const fbl_params *p, 
     }
     if (e == cudaSuccess) e = cudaMalloc(&s->grad, nvox * sizeof(float));
     if (e == cudaSuccess && p->reg == FBL_REG_TV) {
-        // b, y and two dual pairs (q, r) of the TV prox: 14 volumes of FP32
-        e = cudaMalloc(&s->tv_buf, 14 * nvox * sizeof(float));
+        // b and three duals of the TV prox: 10 volumes of FP32
+        e = cudaMalloc(&s->tv_buf, 10 * nvox * sizeof(float));
     }
     if (e == cudaSuccess) e = cudaMalloc(&s->xstage, nvox * es);
     if (e == cudaSuccess) e = cudaMalloc(&s->d_views, (size_t)d.n_views * sizeof(int32_t));

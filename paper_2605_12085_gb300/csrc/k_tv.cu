@@ -8,14 +8,16 @@
 // is computed by the fast gradient projection on the dual of Beck and
 // Teboulle (2009): per inner iteration
 //
-//     y = P_C(b - lambda K^T r)                               (k_tv_primal)
-//     q' = P_ball(r + K y / (12 lambda)),  r = q' + theta (q' - q),  q = q'  (k_tv_dual)
+//     y = P_C(b - lambda K^T r),  r = q + theta (q - q_prev)
+//     q' = P_ball(r + K y / (12 lambda))
 //
-// and the result P_C(b - lambda K^T q).  Both kernels stream the volumes once
-// (memory-bound: 20 and 52 bytes per voxel).  The dual pair (q, r) alternates
-// between two buffers: k_tv_dual reads one pair and writes the other.  (Updated
-// in place -- every thread storing to the six lines it had just loaded -- the
-// same kernel ran 8x slower, its loads waiting ~20 us with DRAM 8% busy.)
+// and the result P_C(b - lambda K^T q).  One kernel does an inner iteration
+// (k_tv_step): it forms r from the last two duals instead of storing it, and
+// y on the fly, so the volumes are streamed once, 40 bytes per voxel (b, q and
+// q_prev read, q' written); the duals rotate through three buffers.  As two
+// kernels with y and r in memory (20 + 52 bytes) an iteration took 1.61 ms at
+// 512^3; the dual updated in place -- every thread storing to the lines it had just
+// loaded -- ran 8x slower than that.
 // Volumes are in any memory order given
 // by (n0 fastest, n1, n2); a dual field is 3 volumes, component c along axis c
 // of that order (the isotropic norm does not depend on the order).  The
@@ -24,6 +26,7 @@
 // the sums of the test (2.3) with the same blocks as the l1 prox, read the
 // z-innermost iterate layout.
 #include <cmath>
+#include <cstdint>
 
 #include "fbl_internal.cuh"
 #include "fbl_reduce.cuh"
@@ -62,49 +65,86 @@ __global__ void __launch_bounds__(TV_NT) k_tv_primal(const float *__restrict__ b
     y[e] = fminf(fmaxf(fmaf(-lam, kt, b[e]), 0.f), xmax);
 }
 
-__global__ void __launch_bounds__(TV_NT) k_tv_dual(const float *__restrict__ y, Dims d, float inv12lam,
-                                                   float theta, const float *__restrict__ q,
-                                                   const float *__restrict__ r, float *__restrict__ qo,
-                                                   float *__restrict__ ro) {
-    const int a0 = blockIdx.x * TV_NT + threadIdx.x, a1 = blockIdx.y, a2 = blockIdx.z;
-    if (a0 >= d.n0) return;
-    const size_t N = d.N(), e = ((size_t)a2 * d.n1 + a1) * d.n0 + a0;
-    const size_t s1 = d.n0, s2 = (size_t)d.n0 * d.n1;
-    const float yv = y[e];
-    // components whose difference does not exist stay zero
-    float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-    const bool h0 = a0 < d.n0 - 1, h1 = a1 < d.n1 - 1, h2 = a2 < d.n2 - 1;
-    if (h0) g0 = fmaf(inv12lam, y[e + 1] - yv, r[e]);
-    if (h1) g1 = fmaf(inv12lam, y[e + s1] - yv, r[N + e]);
-    if (h2) g2 = fmaf(inv12lam, y[e + s2] - yv, r[2 * N + e]);
-    const float nrm = sqrtf(fmaf(g0, g0, fmaf(g1, g1, g2 * g2)));
-    const float sc = 1.f / fmaxf(nrm, 1.f);
-    g0 *= sc;
-    g1 *= sc;
-    g2 *= sc;
-    const float o0 = q[e], o1 = q[N + e], o2 = q[2 * N + e];
-    qo[e] = g0;
-    qo[N + e] = g1;
-    qo[2 * N + e] = g2;
-    ro[e] = fmaf(theta, g0 - o0, g0);
-    ro[N + e] = fmaf(theta, g1 - o1, g1);
-    ro[2 * N + e] = fmaf(theta, g2 - o2, g2);
+// One inner iteration.  A block owns TS_W x TS_H columns of the volume and marches
+// up a2 from blockIdx.z * planes; its 32 x (TS_H + 2) threads cover the columns
+// and one more on every side: y needs the duals of the lower neighbours, the new
+// dual the y of the upper ones.  Per plane a thread loads its voxel's duals and b,
+// exchanges r along a0 by shuffles and along a1 through shared memory, forms y,
+// and finishes the dual of the plane below, whose neighbours' y are known now.
+// HBM-bound: the halo's second reads come from L2 (TS_W = 30 of 32 lanes, 14 of 16
+// rows: 1.22 loads per voxel).
+constexpr int TS_W = 30, TS_H = 14;
+
+__global__ void __launch_bounds__(32 * (TS_H + 2), 4) k_tv_step(const float *__restrict__ b, Dims d, float lam, float xmax,
+                                                                float inv12lam, float theta,
+                                                                const float *__restrict__ q, const float *__restrict__ qp,
+                                                                float *__restrict__ qo, int planes) {
+    __shared__ float s_r1[2][TS_H + 2][32], s_y[2][TS_H + 2][32];
+    const int lane = threadIdx.x, row = threadIdx.y;
+    const int a0 = blockIdx.x * TS_W - 1 + lane, a1 = blockIdx.y * TS_H - 1 + row;
+    const int z0 = blockIdx.z * planes, z1 = min(z0 + planes, d.n2);
+    const bool in = a0 >= 0 && a0 < d.n0 && a1 >= 0 && a1 < d.n1;
+    const bool own = in && lane >= 1 && lane <= TS_W && row >= 1 && row <= TS_H;
+    const size_t N = d.N(), s2 = (size_t)d.n0 * d.n1;
+    size_t e = (size_t)z0 * s2 + (in ? (size_t)a1 * d.n0 + a0 : 0);
+    const bool h0 = a0 < d.n0 - 1, h1 = a1 < d.n1 - 1;
+    auto dual = [&](size_t at) {
+        const float v = q[at];
+        return fmaf(theta, v - qp[at], v);
+    };
+    float r0p = 0.f, r1p = 0.f, r2p = 0.f, yp = 0.f;  // the plane below
+    if (z0 > 0 && in) r2p = dual(2 * N + e - s2);
+    for (int z = z0; z <= z1; ++z, e += s2) {
+        const int buf = z & 1;
+        const bool on = in && z < d.n2;
+        float r0 = 0.f, r1 = 0.f, r2 = 0.f, bv = 0.f;
+        if (on) {
+            r0 = dual(e);
+            r1 = dual(N + e);
+            r2 = dual(2 * N + e);
+            bv = b[e];
+        }
+        s_r1[buf][row][lane] = r1;
+        __syncthreads();
+        const float r0m = __shfl_up_sync(0xffffffffu, r0, 1);
+        // (K^T r)(v), a missing difference's component being zero
+        float kt = 0.f - r0;
+        if (a0 > 0) kt += r0m;
+        kt -= r1;
+        if (a1 > 0 && row > 0) kt += s_r1[buf][row - 1][lane];
+        kt -= r2;
+        kt += r2p;
+        const float y = fminf(fmaxf(fmaf(-lam, kt, bv), 0.f), xmax);
+        s_y[buf][row][lane] = y;
+        // the dual of the plane below
+        const float yp0 = __shfl_down_sync(0xffffffffu, yp, 1);
+        if (own && z > z0) {
+            float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+            if (h0) g0 = fmaf(inv12lam, yp0 - yp, r0p);
+            if (h1) g1 = fmaf(inv12lam, s_y[buf ^ 1][row + 1][lane] - yp, r1p);
+            if (z < d.n2) g2 = fmaf(inv12lam, y - yp, r2p);
+            const float sc = 1.f / fmaxf(sqrtf(fmaf(g0, g0, fmaf(g1, g1, g2 * g2))), 1.f);
+            const size_t o = e - s2;
+            qo[o] = g0 * sc;
+            qo[N + o] = g1 * sc;
+            qo[2 * N + o] = g2 * sc;
+        }
+        r0p = r0;
+        r1p = r1;
+        r2p = r2;
+        yp = y;
+    }
 }
 
-// The starting pair (qo, ro) = (q, q) with q's components without a
-// difference set to zero (q = NULL: both zero).
-__global__ void __launch_bounds__(TV_NT) k_tv_start(Dims d, const float *__restrict__ q, float *__restrict__ qo,
-                                                    float *__restrict__ ro) {
+// The starting dual qo = q with the components without a difference set to
+// zero (q = NULL: zero).
+__global__ void __launch_bounds__(TV_NT) k_tv_start(Dims d, const float *__restrict__ q, float *__restrict__ qo) {
     const int a0 = blockIdx.x * TV_NT + threadIdx.x, a1 = blockIdx.y, a2 = blockIdx.z;
     if (a0 >= d.n0) return;
     const size_t N = d.N(), e = ((size_t)a2 * d.n1 + a1) * d.n0 + a0;
     const bool h[3] = {a0 < d.n0 - 1, a1 < d.n1 - 1, a2 < d.n2 - 1};
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float v = (!q || !h[c]) ? 0.f : q[c * N + e];
-        qo[c * N + e] = v;
-        ro[c * N + e] = v;
-    }
+    for (int c = 0; c < 3; ++c) qo[c * N + e] = (!q || !h[c]) ? 0.f : q[c * N + e];
 }
 
 // Per-block FP64 sums of ||(K x)_v||_2.
@@ -184,20 +224,36 @@ __global__ void __launch_bounds__(TV_TX *TV_TY) k_tv_final_zi(const T *__restric
 
 dim3 tv_grid(const Dims &d) { return dim3((d.n0 + TV_NT - 1) / TV_NT, d.n1, d.n2); }
 
-// FGP iterations from the pair (q[*cur], r[*cur]), alternating between the
-// two pairs; *cur ends at the pair holding the last dual.  theta_k from
-// t_1 = 1, t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2.
-cudaError_t fgp_iterations(const float *b, const Dims &d, float lam, float xmax, int iters, float *y,
-                           float *const q[2], float *const r[2], int *cur, cudaStream_t st) {
-    const dim3 grid = tv_grid(d);
+// FGP iterations from the dual q[*cur], rotating through the three buffers; *cur
+// ends at the last dual.  theta_k from t_1 = 1, t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2
+// (the first iteration's r is q itself).
+cudaError_t fgp_iterations(const float *b, const Dims &d, float lam, float xmax, int iters, float *const q[3], int *cur,
+                           cudaStream_t st) {
     const float inv12 = (float)(1.0 / (12.0 * (double)lam));
+    // planes per block: the fewest planes read (one more than written) over full
+    // waves of 4 blocks per SM
+    const int64_t cols = (int64_t)((d.n0 + TS_W - 1) / TS_W) * ((d.n1 + TS_H - 1) / TS_H);
+    int planes = d.n2;
+    int64_t best = INT64_MAX;
+    for (int c = 1; c <= d.n2 && c <= 64; ++c) {
+        const int p = (d.n2 + c - 1) / c;
+        const int64_t waves = (cols * ((d.n2 + p - 1) / p) + 152 * 4 - 1) / (152 * 4);
+        if (waves * (p + 2) < best) {
+            best = waves * (p + 2);
+            planes = p;
+        }
+    }
+    const dim3 grid((d.n0 + TS_W - 1) / TS_W, (d.n1 + TS_H - 1) / TS_H, (d.n2 + planes - 1) / planes);
     double t = 1.0;
-    int c = *cur;
+    float theta = 0.f;
+    int c = *cur, prev = *cur;
     for (int it = 0; it < iters; ++it) {
+        const int next = it == 0 ? (c + 1) % 3 : 3 - c - prev;
+        k_tv_step<<<grid, dim3(32, TS_H + 2), 0, st>>>(b, d, lam, xmax, inv12, theta, q[c], q[prev], q[next], planes);
         const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
-        k_tv_primal<<<grid, TV_NT, 0, st>>>(b, r[c], d, lam, xmax, y);
-        k_tv_dual<<<grid, TV_NT, 0, st>>>(y, d, inv12, (float)((t - 1.0) / tn), q[c], r[c], q[1 - c], r[1 - c]);
-        c = 1 - c;
+        theta = (float)((t - 1.0) / tn);
+        prev = c;
+        c = next;
         t = tn;
     }
     *cur = c;
@@ -209,14 +265,13 @@ cudaError_t fgp_iterations(const float *b, const Dims &d, float lam, float xmax,
 bool tv_dims_ok(int n0, int n1, int n2) { return n0 > 0 && n1 > 0 && n2 > 0 && n1 <= 65535 && n2 <= 65535; }
 
 cudaError_t launch_tv_prox(const float *v, int n0, int n1, int n2, float lam, float xmax, int iters,
-                           const float *q_start, float *const q[2], float *const r[2], float *y, float *x, int *cur,
-                           cudaStream_t st) {
+                           const float *q_start, float *const q[3], float *x, int *cur, cudaStream_t st) {
     const Dims d{n0, n1, n2};
     const dim3 grid = tv_grid(d);
-    k_tv_start<<<grid, TV_NT, 0, st>>>(d, q_start, q[*cur], r[*cur]);
+    k_tv_start<<<grid, TV_NT, 0, st>>>(d, q_start, q[*cur]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (lam > 0.f && (e = fgp_iterations(v, d, lam, xmax, iters, y, q, r, cur, st)) != cudaSuccess) return e;
+    if (lam > 0.f && (e = fgp_iterations(v, d, lam, xmax, iters, q, cur, st)) != cudaSuccess) return e;
     // result P_C(v - lam K^T q): the primal kernel on q (lam = 0 gives P_C(v))
     k_tv_primal<<<grid, TV_NT, 0, st>>>(v, q[*cur], d, lam > 0.f ? lam : 0.f, xmax, x);
     return cudaGetLastError();
@@ -231,8 +286,8 @@ cudaError_t launch_tv_norm(const float *x, int n0, int n1, int n2, double *parti
 }
 
 cudaError_t launch_tv_prox_zi(const void *vol, ZLayout L, const float *gzi, float alpha, float lam, float xmax,
-                              int iters, int warm, float *b, float *const q[2], float *const r[2], int *cur,
-                              float *y, void *trial, int dtype, double *partials, int *n_partials, cudaStream_t st) {
+                              int iters, int warm, float *b, float *const q[3], int *cur, void *trial, int dtype,
+                              double *partials, int *n_partials, cudaStream_t st) {
     const int nb = (L.nx * L.ny + TV_TY - 1) / TV_TY;
     if (nb != prox_zi_num_partials(L.nx, L.ny, L.nz)) return cudaErrorInvalidConfiguration;
     const dim3 blk(TV_TX, TV_TY);
@@ -242,13 +297,13 @@ cudaError_t launch_tv_prox_zi(const void *vol, ZLayout L, const float *gzi, floa
         case FBL_F16: k_tv_rhs_zi<<<nb, blk, 0, st>>>((const __half *)vol, L, gzi, alpha, b); break;
         default: k_tv_rhs_zi<<<nb, blk, 0, st>>>((const float *)vol, L, gzi, alpha, b); break;
     }
-    // the start goes to the other pair (from the last dual when warm)
+    // the start goes to another buffer (from the last dual when warm)
     const int c0 = *cur;
-    k_tv_start<<<tv_grid(d), TV_NT, 0, st>>>(d, warm ? q[c0] : nullptr, q[1 - c0], r[1 - c0]);
-    *cur = 1 - c0;
+    *cur = (c0 + 1) % 3;
+    k_tv_start<<<tv_grid(d), TV_NT, 0, st>>>(d, warm ? q[c0] : nullptr, q[*cur]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (lam > 0.f && (e = fgp_iterations(b, d, lam, xmax, iters, y, q, r, cur, st)) != cudaSuccess) return e;
+    if (lam > 0.f && (e = fgp_iterations(b, d, lam, xmax, iters, q, cur, st)) != cudaSuccess) return e;
     const float lm = lam > 0.f ? lam : 0.f;
     const float *qf = q[*cur];
     switch (dtype) {
