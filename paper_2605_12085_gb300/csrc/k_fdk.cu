@@ -19,13 +19,16 @@
 // consecutive entries along z and needs no bounds test at the edges.  The
 // block restages its results in shared memory and stores them as float4s.
 // k_fdk_bp (one launch per 32 views; each adds into the volume but the very
-// first, which writes it): a warp owns one (i, j) voxel
-// column and 32 * FDK_KPL voxels along z (lane l: k0 + l + 32 t).  The FP64
-// geometry of a (column, view) pair (detector column and weight, the
-// vertical map k -> v) is formed by one thread -- lane l of the warp takes
-// view s0 + l -- and kept in shared memory for the warp, so FP64 work (slow
-// on this part) costs one thread per pair instead of a whole warp; every lane
-// then interpolates bilinearly in FP32.  Output in [j][i][k] order.
+// first, which writes it): a block owns 8 x 4 voxel columns, a warp 2 x 2 of them
+// and 32 * KPL voxels along z (lane l: k0 + l + 32 q).  The geometry of a (column,
+// view) pair -- detector column and weight, the row coordinate of voxel k0 and the
+// rows per voxel in Q.32 -- is formed by one thread in FP64 (slow on this part: one
+// reciprocal by an FP32 estimate and a Newton step) and kept in shared memory for the
+// warp.  Per voxel and view: a 64-bit add and a funnel shift for the row, two 8-byte
+// loads, the interpolation along the rows as one packed subtraction and FMA, along
+// the columns and into the sum as three operations.  The four voxel columns of a
+// warp and the 32 of a block read the same few detector columns of a view from L1.
+// Output in [j][i][k] order.
 #include <math.h>
 
 #include "fbl_internal.cuh"
@@ -35,9 +38,8 @@ namespace {
 
 constexpr int FDK_ROWS = 8;    // detector rows per filter block
 constexpr int FDK_FT = 256;    // filter block threads
-constexpr int FDK_KPL = 8;     // voxels per lane along z in the backprojection
-constexpr int FDK_WARPS = 8;   // voxel columns (consecutive i) per backprojection block
-constexpr int FDK_VB = 32;     // views whose pair geometry a block forms at once (one per lane)
+constexpr int FDK_WARPS = 8;   // warps per backprojection block: 4 x 2, each 2 x 2 voxel columns
+constexpr int FDK_VB = 16;     // views whose pair geometry a block forms at once
 
 // float2 entries per detector column of the filtered projections: row v at
 // entry v + 2, two zero entries below row 0 and at least two above row nv - 1,
@@ -144,101 +146,110 @@ struct FdkView {
     double c, s, w;  // cos, sin, dtheta / 2
 };
 
-struct FdkPair {
-    int off;          // entry of (column iu0 + 1, row 0) in the view's block
-    float tu, w, dfv; // horizontal weight, (dtheta/2) / U^2, rows per voxel along z
-};
-struct FdkBase {
-    int ib;    // floor of the detector row of voxel k0 + 32 q
-    float fb;  // and its fraction
+struct __align__(16) FdkPair {
+    const float2 *col;  // row 0 of the column pair
+    long long t;        // Q.32 detector row of voxel k0
+    long long dv;       // Q.32 rows per voxel
+    float tu, w;        // horizontal weight; (dtheta/2) / U^2, 0 where the column is off the detector
 };
 
-__global__ void __launch_bounds__(32 * FDK_WARPS, 5) k_fdk_bp(const float2 *__restrict__ qt, const FdkView *views,
-                                                           int n_sel, int nx, int ny, int nz, int nu, int nv,
-                                                           double vx, double vy, double vz, double sod,
-                                                           double inv_du_m, double inv_dv_m, double cu, double cv,
-                                                           int accumulate, float *__restrict__ gzi) {
-    __shared__ FdkPair hp[FDK_WARPS][FDK_VB];
-    __shared__ FdkBase hb[FDK_WARPS][FDK_KPL][FDK_VB];
+// Interpolation between two rows of a column pair: a + f (b - a) on both halves
+// (packed FP32x2, the roundings of two scalar operations).
+__device__ __forceinline__ float2 fdk_lerp2(float f, float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, f, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 f, {%6, %6};\n\t"
+        "sub.rn.f32x2 b, b, a;\n\tfma.rn.f32x2 d, f, b, a;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(f));
+    return d;
+}
+
+// One (column, view) pair added to the lane's voxels.  CLAMP: some voxel's row
+// lies outside [-2, nv]; it is clamped to rows that are zero, with zero followers.
+template <int KPL, bool CLAMP>
+__device__ __forceinline__ void fdk_add(const FdkPair &p, int nv, float (&acc)[KPL]) {
+    const int lane = threadIdx.x;
+    const float2 *col = p.col;
+    const long long dv = p.dv, dv32 = dv << 5;
+    long long t = p.t + (long long)lane * dv;
+    const float tu = p.tu, w = p.w;
+#pragma unroll
+    for (int q = 0; q < KPL; ++q) {
+        int r = fx32_floor(t);
+        if (CLAMP) r = min(max(r, -2), nv);
+        const float2 A = __ldg(col + r), B = __ldg(col + r + 1);
+        const float2 v = fdk_lerp2(fx32_frac(t), A, B);
+        acc[q] = fmaf(w, fmaf(tu, v.y - v.x, v.x), acc[q]);
+        t += dv32;
+    }
+}
+
+template <int KPL>
+__global__ void __launch_bounds__(32 * FDK_WARPS, 3) k_fdk_bp(const float2 *__restrict__ qt, const FdkView *views, int n_sel,
+                                                           int nx, int ny, int nz, int nu, int nv, double vx, double vy,
+                                                           double sod, double inv_du_m, double rows_per_voxel, double cu,
+                                                           double cv, int accumulate, float *__restrict__ gzi) {
+    __shared__ FdkPair pairs[FDK_WARPS][FDK_VB][4];
     const int lane = threadIdx.x, wi = threadIdx.y;
-    const int i = blockIdx.x * FDK_WARPS + wi, j = blockIdx.y;
-    const int k0 = blockIdx.z * 32 * FDK_KPL;
-    const bool col = i < nx;  // columns past nx still take part in the barriers
-    const double x = (i - 0.5 * (nx - 1)) * vx, yy = (j - 0.5 * (ny - 1)) * vy;
-    const double czk = 0.5 * (nz - 1);
+    const int i0 = blockIdx.x * 8 + 2 * (wi & 3), j0 = blockIdx.y * 4 + 2 * (wi >> 2);
+    const int k0 = blockIdx.z * 32 * KPL;
     const int rs = fdk_row_stride(nv);
     const size_t vstride = (size_t)(nu + 1) * rs;
-    float acc[FDK_KPL];
+    float acc[4][KPL];
 #pragma unroll
-    for (int q = 0; q < FDK_KPL; ++q) acc[q] = 0.f;
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int q = 0; q < KPL; ++q) acc[c][q] = 0.f;
     for (int s0 = 0; s0 < n_sel; s0 += FDK_VB) {
         const int nb = min(FDK_VB, n_sel - s0);
-        if (lane < nb) {
-            const FdkView v = views[s0 + lane];
-            const double xi = x * v.c + yy * v.s, eta = -x * v.s + yy * v.c;
-            const double invU = sod / (sod - xi);
-            const double fu = eta * invU * inv_du_m + cu;
-            // a column that projects off the detector reads column 0 with
-            // weight 0 and rows that fail the range test below
-            FdkPair p{2, 0.f, 0.f, 0.f};
-            const bool on = fu > -1.0 && fu < (double)nu;
-            const double dfv = vz * invU * inv_dv_m;
-            if (on) {
-                const double fl = floor(fu);
-                p.off = ((int)fl + 1) * rs + 2;
-                p.tu = (float)(fu - fl);
+        __syncwarp();
+        // half a warp per voxel column, a view per lane
+        for (int h = 0; h < 2; ++h) {
+            const int c = 2 * h + (lane >> 4), sv = lane & 15;
+            if (sv >= nb) continue;
+            const FdkView v = views[s0 + sv];
+            const double x = (i0 + (c & 1) - 0.5 * (nx - 1)) * vx, y = (j0 + (c >> 1) - 0.5 * (ny - 1)) * vy;
+            const double D = sod - fma(x, v.c, y * v.s);
+            // 1 / D: an FP32 estimate and one Newton step (relative error 2^-45)
+            const double e0 = (double)__frcp_rn((float)D), inv = fma(e0, fma(-D, e0, 1.0), e0);
+            const double invU = sod * inv;
+            const double fu = fma(fma(y, v.c, -x * v.s) * invU, inv_du_m, cu);
+            const double dfv = rows_per_voxel * invU;
+            FdkPair p;
+            p.col = qt;
+            p.t = p.dv = 0;
+            p.tu = p.w = 0.f;
+            const bool in = i0 + (c & 1) < nx && j0 + (c >> 1) < ny;
+            if (in && fu > -1.0 && fu < (double)nu) {
+                const long long F = __double2ll_rd(fu * 4294967296.0);
+                p.col = qt + (size_t)(s0 + sv) * vstride + (size_t)(fx32_floor(F) + 1) * rs + 2;
+                p.tu = fx32_frac(F);
                 p.w = (float)(v.w * invU * invU);
-                p.dfv = (float)dfv;
+                p.dv = __double2ll_rn(dfv * 4294967296.0);
+                p.t = __double2ll_rn(fma(k0 - 0.5 * (nz - 1), dfv, cv) * 4294967296.0);
             }
-            // detector row of voxel k: fv0 + k * dfv, as a base per 32 voxels in
-            // Q32 fixed point (error <= 2^-33 (1 + 32 q) rows from rounding the
-            // start and the step) plus a small FP32 offset per lane: integer
-            // steps instead of FP64 ones per base
-            const double fv0 = cv - czk * dfv;
-            const long long D = __double2ll_rn(dfv * 4294967296.0);
-            long long B = __double2ll_rn((fv0 + (double)k0 * dfv) * 4294967296.0);
-#pragma unroll
-            for (int q = 0; q < FDK_KPL; ++q, B += 32 * D) {
-                const int ib = (int)(B >> 32);
-                const float fb = (float)(unsigned)(B & 0xffffffffLL) * 2.3283064365386963e-10f;  // 2^-32
-                hb[wi][q][lane] = on ? FdkBase{ib, fb} : FdkBase{-(1 << 30), 0.f};
-            }
-            hp[wi][lane] = p;
+            pairs[wi][sv][c] = p;
         }
-        __syncthreads();
-        if (col) {
-#pragma unroll 2
-            for (int t = 0; t < nb; ++t) {
-                const FdkPair p = hp[wi][t];
-                const float2 *col2 = qt + (size_t)(s0 + t) * vstride + p.off;
-                const float lf = (float)lane * p.dfv;  // |.| <= 31 dfv
+        __syncwarp();
+        for (int t = 0; t < nb; ++t) {
 #pragma unroll
-                for (int q = 0; q < FDK_KPL; ++q) {
-                    const FdkBase bb = hb[wi][q][t];
-                    const float fl = bb.fb + lf;
-                    const float fll = floorf(fl);
-                    const int iv0 = bb.ib + (int)fll;
-                    // taps clamped into the column so the loads need no branch;
-                    // a voxel whose rows fall off the detector keeps its sum
-                    // (lanes past nz accumulate values that are never stored)
-                    const bool ok = iv0 >= -1 && iv0 <= nv - 1;
-                    const int ivc = min(max(iv0, -1), nv - 1);
-                    const float tv = fl - fll;
-                    const float2 A = __ldg(col2 + ivc), B = __ldg(col2 + ivc + 1);  // rows iv0, iv0 + 1
-                    const float lo = fmaf(tv, B.x - A.x, A.x), hi = fmaf(tv, B.y - A.y, A.y);
-                    const float nxt = fmaf(p.w, fmaf(p.tu, hi - lo, lo), acc[q]);
-                    acc[q] = ok ? nxt : acc[q];
-                }
+            for (int c = 0; c < 4; ++c) {
+                const FdkPair &p = pairs[wi][t][c];
+                if (p.w == 0.f) continue;  // uniform over the warp
+                if (fx32_floor(p.t) >= -2 && fx32_floor(p.t + (32 * KPL - 1) * p.dv) <= nv) fdk_add<KPL, false>(p, nv, acc[c]);
+                else fdk_add<KPL, true>(p, nv, acc[c]);
             }
         }
-        __syncthreads();
     }
-    if (!col) return;
-    float *out = gzi + ((size_t)j * nx + i) * nz;
 #pragma unroll
-    for (int q = 0; q < FDK_KPL; ++q) {
-        const int k = k0 + lane + 32 * q;
-        if (k < nz) out[k] = accumulate ? out[k] + acc[q] : acc[q];
+    for (int c = 0; c < 4; ++c) {
+        const int i = i0 + (c & 1), j = j0 + (c >> 1);
+        if (i >= nx || j >= ny) continue;
+        float *out = gzi + ((size_t)j * nx + i) * nz;
+#pragma unroll
+        for (int q = 0; q < KPL; ++q) {
+            const int k = k0 + lane + 32 * q;
+            if (k < nz) out[k] = accumulate ? out[k] + acc[c][q] : acc[c][q];
+        }
     }
 }
 
@@ -289,15 +300,20 @@ cudaError_t launch_fdk_bp(const float *qt, const double *view_csw, int n_sel, in
                           int nv, double vx, double vy, double vz, double sod, double sdd, double du, double dv,
                           int accumulate, float *gzi, cudaStream_t st) {
     const double m = sod / sdd;
+    // voxels per lane: the least work over the spans of 32 KPL voxels
+    int kpl = 8;
+    const auto cost = [nz](int k) { return ((nz + 32 * k - 1) / (32 * k)) * (k + 1); };
+    for (int k : {6, 4, 2})
+        if (cost(k) < cost(kpl)) kpl = k;
     dim3 block(32, FDK_WARPS);
-    dim3 grid((nx + FDK_WARPS - 1) / FDK_WARPS, ny, (nz + 32 * FDK_KPL - 1) / (32 * FDK_KPL));
+    dim3 grid((nx + 7) / 8, (ny + 3) / 4, (nz + 32 * kpl - 1) / (32 * kpl));
     const size_t vstride = (size_t)(nu + 1) * fdk_row_stride(nv);  // float2 entries per view
+    auto kernel = kpl == 8 ? k_fdk_bp<8> : kpl == 6 ? k_fdk_bp<6> : kpl == 4 ? k_fdk_bp<4> : k_fdk_bp<2>;
     for (int s0 = 0; s0 < n_sel; s0 += FDK_SUB) {
         const int ns = n_sel - s0 < FDK_SUB ? n_sel - s0 : FDK_SUB;
-        k_fdk_bp<<<grid, block, 0, st>>>((const float2 *)qt + (size_t)s0 * vstride,
-                                         (const FdkView *)view_csw + s0, ns, nx, ny, nz, nu, nv, vx, vy, vz, sod,
-                                         1.0 / (du * m), 1.0 / (dv * m), 0.5 * (nu - 1), 0.5 * (nv - 1),
-                                         (accumulate || s0 > 0) ? 1 : 0, gzi);
+        kernel<<<grid, block, 0, st>>>((const float2 *)qt + (size_t)s0 * vstride, (const FdkView *)view_csw + s0, ns, nx,
+                                       ny, nz, nu, nv, vx, vy, sod, 1.0 / (du * m), vz / (dv * m), 0.5 * (nu - 1),
+                                       0.5 * (nv - 1), (accumulate || s0 > 0) ? 1 : 0, gzi);
     }
     return cudaGetLastError();
 }
