@@ -194,6 +194,7 @@ struct BpArgs {
     float scale;
     float *gzi;
     double *g2_partials;  // optional: per-block sum of the squared gradient
+    int more, last;       // strips: add to gzi's sums; scale the sum (and form its squares)
 };
 // The backprojector in strips (k_strips.cu): blocks of STRIP_EDGE x STRIP_EDGE
 // voxel columns and 32 strip_zp voxels along z.  A span of 32 ZP voxels costs

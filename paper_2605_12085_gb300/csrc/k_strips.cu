@@ -465,13 +465,12 @@ __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int 
                 for (int q = 0; q < ZP; ++q) {
                     const int k = kb + lane + 32 * q;
                     if (k < g.nz) {
-                        if (fam) {
-                            out[k] = C[q];
-                        } else {
-                            const float val = a.scale * (out[k] + C[q]);
-                            out[k] = val;
+                        float val = fam && !a.more ? C[q] : out[k] + C[q];
+                        if (!fam && a.last) {
+                            val *= a.scale;
                             g2 = fmaf(val, val, g2);
                         }
+                        out[k] = val;
                     }
                 }
             }
@@ -531,6 +530,8 @@ __global__ void __launch_bounds__(32 * KBS_WARPS, 5) kb_strips(const BatchHdr *h
             sa.scale = bv.scale;
             sa.gzi = bv.grad;
             sa.g2_partials = bv.partials;
+            sa.more = 0;
+            sa.last = 1;
         }
         __syncthreads();
         const BpArgs &a = sa;
@@ -563,11 +564,27 @@ cudaError_t launch_batch_strips(const BatchHdr *hdr, BatchVol *vols, int *ctr, c
     return cudaGetLastError();
 }
 
+// Views a launch takes at most: 512 MiB of residual rows.  The blocks of a launch
+// walk its views in order but drift apart; over 1.7 GB of rows (720 views at 512^3)
+// the re-reads from DRAM cost more than adding into the gradient again (107 ms in one
+// launch, 91 in four), up to 0.5 GB they do not (720 views at 256^3: 12.3 ms in one
+// launch, 13.4 in five; 200 at 512^3: 24.7 and 24.8).
+constexpr size_t STRIP_BYTES = size_t(512) << 20;
+
 cudaError_t launch_strips(const BpArgs &a, dim3 grid, int zp, cudaStream_t st) {
-    switch (zp) {
-        case 4: k2_strips<4><<<grid, 32 * STRIP_EDGE, 0, st>>>(a); break;
-        case 6: k2_strips<6><<<grid, 32 * STRIP_EDGE, 0, st>>>(a); break;
-        default: k2_strips<8><<<grid, 32 * STRIP_EDGE, 0, st>>>(a); break;
+    auto k = zp == 4 ? k2_strips<4> : zp == 6 ? k2_strips<6> : k2_strips<8>;
+    const size_t bytes = (size_t)a.n_sel * a.g.nu * rt_pitch(a.g.nv) * sizeof(float);
+    const int parts = (int)std::min((bytes + STRIP_BYTES - 1) / STRIP_BYTES, (size_t)std::max(1, a.n_sel));
+    for (int p = 0; p < parts; ++p) {
+        const int s0 = (int)((int64_t)a.n_sel * p / parts), s1 = (int)((int64_t)a.n_sel * (p + 1) / parts);
+        BpArgs b = a;
+        b.rt = a.rt + (size_t)s0 * a.g.nu * rt_pitch(a.g.nv);
+        b.views = a.views + s0;
+        b.n_sel = s1 - s0;
+        b.more = p > 0;
+        b.last = p + 1 == parts;
+        if (!b.last) b.g2_partials = nullptr;
+        k<<<grid, 32 * STRIP_EDGE, 0, st>>>(b);
     }
     return cudaGetLastError();
 }

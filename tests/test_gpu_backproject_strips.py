@@ -67,3 +67,21 @@ def test_batch_of_columns_and_strips_equals_single_solvers():
         for _ in range(3):
             S.step(x, b)
         assert np.array_equal(host(x), host(xb))
+
+
+def test_views_beyond_one_launch_are_added():
+    # more than 512 MiB of residual rows run in several launches: the same sums as
+    # two calls of one launch each (FP32 sums in another order: 1e-6)
+    import torch
+    import paper_2605_12085_gb300 as fbl
+    g = synth.Geometry(nx=40, ny=33, nz=70, vx=1.0, vy=1.0, vz=1.0, n_views=720, sod=400.0, sdd=700.0, nu=520, nv=400,
+                       du=0.25, dv=0.5)
+    G = fbl.geometry_create(g)
+    fbl.geometry_set_launch(G, 8, 1, 28)
+    gen = torch.Generator("cuda").manual_seed(2)
+    y = torch.rand((720, 400, 520), device="cuda", generator=gen)
+    views = list(range(720))
+    x = fbl.backproject(G, y, views)
+    two = fbl.backproject(G, y[:300].contiguous(), views[:300])
+    fbl.backproject(G, y[300:].contiguous(), views[300:], x=two, accumulate=True)
+    assert rel_l2(host(x), host(two)) <= 1e-6
