@@ -352,8 +352,11 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
     dg.inv_du = (float)(1.0 / d.du);
     dg.hwu = (float)hw;
     dg.cz_fx = (long long)std::llround(cxyz[2] * FX_ONE);
-    dg.k1_cols = 8;
-    dg.k1_split = 1;
+    // 4 columns per block, plain plane loop: the fastest or within 1 % of it at every
+    // size measured (objective of 10 views at 64^3 13.6 us, 20 at 256^3 0.328 ms, 40 at
+    // 512^3 5.13; with 8 columns and loads one sample ahead 15.7, 0.357, 5.38)
+    dg.k1_cols = 4;
+    dg.k1_split = 0;
     dg.k2_vpl = backproject_default_config(d.nx, d.ny, d.nz);
     // detector rows with a crossing in (k - 1, k + 1) on one column: at most
     // floor(2 max_inv) + 1

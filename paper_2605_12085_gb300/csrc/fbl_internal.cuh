@@ -129,7 +129,7 @@ struct DevGeom {
     float sod, sdd, inv_du;
     float hwu;                   // half width, in columns, of a voxel's column footprint
     int ntap;                    // detector rows that can touch one voxel in one column
-    // launch configuration (by the autotuner; defaults 8 / 1 / by the volume's size)
+    // launch configuration (by the autotuner; defaults 4 / 0 / by the volume's size)
     int k1_cols;                 // projector: detector columns per block (4 or 8)
     int k1_split;                // projector plane loop: 0 plain, 1 loads one sample ahead, 2 TMA-staged bricks
     int k2_vpl;                  // backprojector: voxel columns (2, 4, 24) or strips (8, 16, 28)

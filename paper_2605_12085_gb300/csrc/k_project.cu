@@ -153,8 +153,7 @@ __device__ __forceinline__ void chunk_loop(const TX *__restrict__ vol, const int
     struct Smp {
         float v00, v10, v01, v11, fb, fz;
     };
-    auto fetch = [&](int j, Smp &o) {
-        const int2 e = tab[j];
+    auto fetch = [&](const int2 &e, Smp &o) {
         // qz carries +2: k0 + 2 as unsigned, clamped to nz + 2 (rows below -2
         // wrap to the top: both ends hold two zero elements); e.x carries -2
         const unsigned k2 = min((unsigned)fx32_floor(qz), (unsigned)(nz + 2));
@@ -176,31 +175,35 @@ __device__ __forceinline__ void chunk_loop(const TX *__restrict__ vol, const int
         int j = 0;
 #pragma unroll 1
         for (; j + 1 < len; j += 2) {
+            // two entries in one 16-byte broadcast: shared-memory reads are a fifth of
+            // the kernel's L1 wavefronts (20 views at 256^3: 0.340 -> 0.328 ms); with the
+            // loads one sample ahead the extra registers cost more than that
+            const int4 e = *reinterpret_cast<const int4 *>(tab + j);
             Smp a, b;
-            fetch(j, a);
-            fetch(j + 1, b);
+            fetch(make_int2(e.x, e.y), a);
+            fetch(make_int2(e.z, e.w), b);
             s0 += value(a);
             s1 += value(b);
         }
         if (j < len) {
             Smp a;
-            fetch(j, a);
+            fetch(tab[j], a);
             s0 += value(a);
         }
         return;
     }
     Smp a, b;
-    fetch(0, a);
+    fetch(tab[0], a);
     int j = 0;
 #pragma unroll 1
     for (; j + 2 < len; j += 2) {
-        fetch(j + 1, b);
+        fetch(tab[j + 1], b);
         s0 += value(a);
-        fetch(j + 2, a);
+        fetch(tab[j + 2], a);
         s1 += value(b);
     }
     if (j + 1 < len) {
-        fetch(j + 1, b);
+        fetch(tab[j + 1], b);
         s0 += value(a);
         s1 += value(b);
     } else {
@@ -271,7 +274,7 @@ __device__ __forceinline__ void epilogue(const ProjArgs &a, const float4 &cB, in
 // each sample's loads one sample ahead (launch configuration k1_split = 1).
 template <typename TX, typename TB, typename TO, int MODE, int COLS, bool PIPE>
 __device__ __forceinline__ void k1_tile(const ProjArgs &a, int cb, int s, int band, double *partial) {
-    __shared__ int2 tab_all[COLS][K1_CHUNK];
+    __shared__ __align__(16) int2 tab_all[COLS][K1_CHUNK];
     const DevGeom &g = a.g;
     const int lane = threadIdx.x;
     const int iu = cb * COLS + threadIdx.y;  // uniform over the warp
