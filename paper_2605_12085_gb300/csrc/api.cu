@@ -533,8 +533,7 @@ fbl_status pack_volume(const fbl_geometry *g, const void *xdev, int dtype, Async
     L = layout_for(g, dtype);
     const size_t bytes = (size_t)L.elems() * dtype_size(dtype);
     CK(pv.alloc(bytes, st), "volume layout");
-    CK(cudaMemsetAsync(pv.p, 0, bytes, st), "memset");
-    CK(launch_pack(xdev, dtype, pv.p, L, st), "pack");
+    CK(launch_pack(xdev, dtype, pv.p, L, true, st), "pack");
     return FBL_OK;
 }
 
@@ -1509,7 +1508,7 @@ fbl_status solver_load_x(fbl_solver *s, const void *x, bool x_dev, cudaStream_t 
         src = s->xstage;
     }
     CK(prof_launch(s, 5, st, [&] {
-           return launch_pack(src, s->p.x_dtype, s->st, s->L, st);
+           return launch_pack(src, s->p.x_dtype, s->st, s->L, false, st);
        }),
        "pack");
     return FBL_OK;

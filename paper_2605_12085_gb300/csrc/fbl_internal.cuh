@@ -145,8 +145,8 @@ enum ProjMode { PROJ_STORE = 0, PROJ_RESID = 1, PROJ_NORM = 2 };
 
 // Kernel launchers (each returns the launch error, if any).
 
-// Natural [nz][ny][nx] volume -> the library layout (interior only).
-cudaError_t launch_pack(const void *x, int x_dtype, void *vol, ZLayout L, cudaStream_t st);
+// Natural [nz][ny][nx] volume -> the library layout (the interior, or with its zero border).
+cudaError_t launch_pack(const void *x, int x_dtype, void *vol, ZLayout L, bool border, cudaStream_t st);
 // Library layout -> natural [nz][ny][nx] (same dtype).
 cudaError_t launch_unpack(const void *vol, ZLayout L, int dtype, void *x, cudaStream_t st);
 // Gradient order [j][i][k] (float) -> natural [nz][ny][nx] float, = or +=.

@@ -325,9 +325,9 @@ __device__ __forceinline__ void k1_tile(const ProjArgs &a, int cb, int s, int ba
                     tab[lane] = make_int2(base - 2 + m * ps + fx_floor(qb) * bs, __float_as_int(fx_frac(qb)));
                 }
                 __syncwarp();
-                // the store mode always issues loads one sample ahead; the residual
-                // and objective modes when the launch configuration asks (PIPE)
-                chunk_loop<MODE == PROJ_STORE || PIPE, TX>(vol, tab, len, bs, g.nz, qz, qz1, s0, s1);
+                // the store mode issues loads one sample ahead for FP32 volumes; the
+                // residual and objective modes when the launch configuration asks (PIPE)
+                chunk_loop<MODE == PROJ_STORE ? sizeof(TX) == 4 : PIPE, TX>(vol, tab, len, bs, g.nz, qz, qz1, s0, s1);
                 __syncwarp();
             }
             acc = s0 + s1;

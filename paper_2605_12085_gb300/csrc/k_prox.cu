@@ -21,12 +21,31 @@ constexpr int TR = 8;         // tile rows per pass
 constexpr int P_NT = TB * TR; // threads per block
 
 // Natural [nz][ny][nx] volume -> the library layout.  For each j, a
-// 32 x 32 (k, i) tile is read along i and written along k.
-template <typename T>
+// 32 x 32 (k, i) tile is read along i and written along k.  BORDER: the zero
+// border too (a fresh buffer; one launch and one pass less than clearing all of it
+// first): the tiles then cover the rows i, j = -1 .. n and the whole pitch.
+template <typename T, bool BORDER>
 __global__ void __launch_bounds__(P_NT) k_pack(const T *__restrict__ x, T *__restrict__ vol,
                                                ZLayout L) {
     __shared__ T tile[TB][TB + 1];  // [k][i]
     const int i0 = blockIdx.x * TB, k0 = blockIdx.y * TB, j = blockIdx.z;
+    if (BORDER) {
+        const int ib = i0 - 1, kb = k0 - L.PL, jb = j - 1;  // row (ib + .., jb), elements from kb on
+        const int tx = threadIdx.x, ty = threadIdx.y;
+#pragma unroll
+        for (int r = 0; r < TB / TR; ++r) {
+            const int k = kb + ty + TR * r, i = ib + tx;
+            const bool in = i >= 0 && i < L.nx && jb >= 0 && jb < L.ny && k >= 0 && k < L.nz;
+            tile[ty + TR * r][tx] = in ? x[((size_t)k * L.ny + jb) * L.nx + i] : from_f32<T>(0.f);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < TB / TR; ++r) {
+            const int i = ib + ty + TR * r, k = kb + tx;
+            if (i <= L.nx && k < L.pitch - L.PL) vol[L.index(i, jb, k)] = tile[tx][ty + TR * r];
+        }
+        return;
+    }
     const int tx = threadIdx.x, ty = threadIdx.y;
 #pragma unroll
     for (int r = 0; r < TB / TR; ++r) {
@@ -267,15 +286,28 @@ __global__ void __launch_bounds__(R_NT) kb_reduce(const BatchVol *vols, int ph, 
 
 }  // namespace
 
-cudaError_t launch_pack(const void *x, int x_dtype, void *vol, ZLayout L, cudaStream_t st) {
-    dim3 block(TB, TR);
-    dim3 grid((L.nx + TB - 1) / TB, (L.nz + TB - 1) / TB, L.ny);
+template <typename T>
+static void pack_t(const void *x, void *vol, const ZLayout &L, bool border, cudaStream_t st) {
+    const dim3 block(TB, TR);
+    if (border)
+        k_pack<T, true><<<dim3((L.nx + 2 + TB - 1) / TB, (L.pitch + TB - 1) / TB, L.ny + 2), block, 0, st>>>(
+            (const T *)x, (T *)vol, L);
+    else
+        k_pack<T, false><<<dim3((L.nx + TB - 1) / TB, (L.nz + TB - 1) / TB, L.ny), block, 0, st>>>((const T *)x,
+                                                                                                (T *)vol, L);
+}
+
+cudaError_t launch_pack(const void *x, int x_dtype, void *vol, ZLayout L, bool border, cudaStream_t st) {
+    // (the border takes two more rows j: past the grid's limit they are cleared first)
+    if (border && (L.ny + 2 > 65535 || (L.pitch + TB - 1) / TB > 65535)) {
+        cudaError_t e = cudaMemsetAsync(vol, 0, (size_t)L.elems() * dtype_size(x_dtype), st);
+        if (e != cudaSuccess) return e;
+        border = false;
+    }
     switch (x_dtype) {
-        case FBL_BF16:
-            k_pack<<<grid, block, 0, st>>>((const __nv_bfloat16 *)x, (__nv_bfloat16 *)vol, L);
-            break;
-        case FBL_F16: k_pack<<<grid, block, 0, st>>>((const __half *)x, (__half *)vol, L); break;
-        default: k_pack<<<grid, block, 0, st>>>((const float *)x, (float *)vol, L); break;
+        case FBL_BF16: pack_t<__nv_bfloat16>(x, vol, L, border, st); break;
+        case FBL_F16: pack_t<__half>(x, vol, L, border, st); break;
+        default: pack_t<float>(x, vol, L, border, st); break;
     }
     return cudaGetLastError();
 }
