@@ -673,7 +673,6 @@ extern "C" fbl_status backproject(const fbl_geometry *g, const void *y, int32_t 
         if ((st = device_input(y, ny_in * dtype_size(y_dtype), ys, &yd, s))) return st;
         const size_t rt_elems = (size_t)n_sel * d.nu * rt_pitch(d.nv);
         CK(rt.alloc(rt_elems * sizeof(float), s), "weighted sinogram");
-        CK(cudaMemsetAsync(rt.p, 0, rt_elems * sizeof(float), s), "memset");
         CK(launch_weight(g->dg, yd, y_dtype, (const int32_t *)dviews.p, n_sel, (float *)rt.p, s),
            "weight kernel");
         CK(gz.alloc(nvox * sizeof(float), s), "gradient scratch");

@@ -172,8 +172,8 @@ int project_num_partials(const DevGeom &g, int n_sel);
 // views, 2 us a trial.)
 bool project_may_stop(const DevGeom &g, int n_sel);
 
-// rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu] (the row weight folded in for K2);
-// the pad entries are left untouched (the caller zeroes them once).
+// rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu] (the row weight folded in for K2),
+// and the rows' zero pads.
 cudaError_t launch_weight(const DevGeom &g, const void *y, int y_dtype, const int32_t *views,
                           int n_sel, float *rt, cudaStream_t st);
 

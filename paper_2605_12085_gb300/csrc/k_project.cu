@@ -745,8 +745,8 @@ __global__ void __launch_bounds__(32 * COLS, 48 / COLS) kb_project(const BatchHd
     }
 }
 
-// rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu], through a 32 x 32 shared tile
-// (reads along iu, writes along iv).
+// rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu] and the rows' zero pads, through a
+// 32 x 32 shared tile (reads along iu, writes along iv).
 template <typename TY>
 __global__ void __launch_bounds__(256) k_weight(const DevGeom g, const TY *__restrict__ y,
                                                 const int32_t *views, float *__restrict__ rt) {
@@ -769,8 +769,11 @@ __global__ void __launch_bounds__(256) k_weight(const DevGeom g, const TY *__res
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int iu = iu0 + ty + 8 * r, iv = iv0 + tx;
-        if (iu < g.nu && iv < g.nv)
-            rt[((size_t)s * g.nu + iu) * rt_pitch(g.nv) + RT_PAD + iv] = tile[tx][ty + 8 * r];
+        float *row = rt + ((size_t)s * g.nu + iu) * rt_pitch(g.nv);
+        if (iu < g.nu && iv < g.nv) row[RT_PAD + iv] = tile[tx][ty + 8 * r];
+        // the zero pads at either end of the row
+        if (iu < g.nu && tx < RT_PAD && iv0 == 0) row[tx] = 0.f;
+        if (iu < g.nu && tx < RT_PAD && iv0 + 32 >= g.nv) row[RT_PAD + g.nv + tx] = 0.f;
     }
 }
 
