@@ -9,8 +9,10 @@
 //
 // Two forms.  Volumes large enough to fill the GPU run in strips (k_strips.cu).
 // Smaller ones run here, one voxel column per warp: many more and shorter warps
-// (64^3, 10 views: 23.9 against 36 us; 16 volumes of 24^3..80^3 in a batch: 0.82
-// against 0.94 ms per iteration).
+// (64^3, 10 views: 23.9 against 36 us).  A batch runs each volume in its own
+// geometry's form, so that its results are the single-volume solver's, although
+// a batch of small volumes fills the GPU and strips would be a little faster there
+// (16 volumes of 24^3..80^3: 0.95 against 1.01 ms per iteration).
 //
 // A warp owns 32*VPL voxels of one (i, j) column along z (lane l holds the VPL
 // consecutive voxels k0 + VPL*l ..; VPL = 2 or 4).  Everything that depends only on (i, j)

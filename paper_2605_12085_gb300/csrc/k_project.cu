@@ -176,7 +176,7 @@ __device__ __forceinline__ void chunk_loop(const TX *__restrict__ vol, const int
 #pragma unroll 1
         for (; j + 1 < len; j += 2) {
             // two entries in one 16-byte broadcast: shared-memory reads are a fifth of
-            // the kernel's L1 wavefronts (20 views at 256^3: 0.340 -> 0.328 ms); with the
+            // the kernel's L1 wavefronts (20 views at 256^3: 0.339 -> 0.328 ms); with the
             // loads one sample ahead the extra registers cost more than that
             const int4 e = *reinterpret_cast<const int4 *>(tab + j);
             Smp a, b;

@@ -38,9 +38,10 @@
 // Measured (40 views at 512^3, 768^2; CUDA events): 8.23 ms for the 2 x 2 groups
 // at 44.5 warp instructions per 32 voxel-views; 7.58 with strips and their sums in
 // registers (36.3); 5.76 with one FMA per weight and 8 voxels per lane (23.1);
-// 5.06 with the sums in tensor memory and 4 blocks per SM; 4.79 with the
+// 5.06 with the sums in tensor memory and 4 blocks per SM; 4.83 with the
 // multiply-add position and the views of the other family dropped by a vote
-// (21.0).  All 720 views: 161 -> 106 ms.  What bounds it now: instruction issue is
+// (21.0).  All 720 views through backproject(): 165.6 -> 111.0 ms, 91 in several
+// launches (see launch_strips).  What bounds it now: instruction issue is
 // active 56 % of cycles, L1 throughput 61 % (three loads per voxel), the rest
 // are load and fixed latencies of 24 to 32 warps per SM.  Not kept: prefetching
 // the next profile's rows or constants (5.1 to 5.5 ms), partial sums ended at
@@ -504,8 +505,9 @@ __global__ void __launch_bounds__(32 * STRIP_EDGE, 4) k2_strips(const BpArgs a) 
 // first `total` tiles of the phase), taken from an atomic counter.  Each volume
 // keeps its own voxels per lane (a block-uniform switch), so its sums are those
 // of its single-volume launch; a block is 4 warps, which take two planes each.
-constexpr int KBS_WARPS = 4;
-__global__ void __launch_bounds__(32 * KBS_WARPS, 5) kb_strips(const BatchHdr *hdr, const BatchVol *vols, int *ctr) {
+constexpr int KBS_WARPS = 4, KBS_BLOCKS = 5;
+static_assert(KBS_BLOCKS * tm_cols(KBS_WARPS, STRIP_EDGE, 8) <= 512, "tensor memory of an SM");
+__global__ void __launch_bounds__(32 * KBS_WARPS, KBS_BLOCKS) kb_strips(const BatchHdr *hdr, const BatchVol *vols, int *ctr) {
     __shared__ int s_tile;
     __shared__ BpArgs sa;
     __shared__ K2Smem<KBS_WARPS> sm;
@@ -552,13 +554,17 @@ __global__ void __launch_bounds__(32 * KBS_WARPS, 5) kb_strips(const BatchHdr *h
 
 }  // namespace
 
+// As many blocks per SM as the launch bound admits (registers, shared memory and
+// 64 of the 512 tensor-memory columns each).  The occupancy query is no guide: it
+// answers 1 for a kernel that allocates tensor memory, and one block per SM took
+// 51.6 ms per iteration of 16 volumes of 96^3 .. 320^3 (learned steps), three
+// 30.5, five 26.5.  No block waits for another, so fewer resident ones are safe.
 cudaError_t launch_batch_strips(const BatchHdr *hdr, BatchVol *vols, int *ctr, cudaStream_t st) {
     static const int grid = [] {
-        int dev = 0, sms = 0, per_sm = 0;
+        int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_strips, 32 * KBS_WARPS, 0);
-        return (sms > 0 ? sms : 1) * std::min(512 / tm_cols(KBS_WARPS, STRIP_EDGE, 8), per_sm > 0 ? per_sm : 1);
+        return (sms > 0 ? sms : 1) * KBS_BLOCKS;
     }();
     kb_strips<<<grid, 32 * KBS_WARPS, 0, st>>>(hdr, vols, ctr);
     return cudaGetLastError();
