@@ -503,10 +503,9 @@ def fdk_record(fbl, G, g, b, xt, device, reps=2):
 
 def regularisers_record(fbl, G, g, b, xt, device, peaks, iters=4):
     """The other regularisers at the workload's size: prox_tv alone (20 FGP
-    iterations on a volume, its algorithmic HBM bytes: 24 B/voxel to start the
-    dual, 72 B/voxel per iteration (20 for y = P_C(b - lam K^T r), 52 for the
-    dual step), 20 B/voxel for the result) against the measured copy
-    bandwidth; and FB-LISA iterations with R = mu||x||_1 + box and with
+    iterations on a volume, its algorithmic HBM bytes: 12 B/voxel to start the
+    dual, 40 B/voxel per iteration (b and two duals read, one dual written),
+    20 B/voxel for the result) against the measured copy bandwidth; and FB-LISA iterations with R = mu||x||_1 + box and with
     R = mu TV + box (10 FGP iterations per prox), ms per iteration from CUDA
     events, beside the paper's R."""
     import torch
@@ -528,7 +527,7 @@ def regularisers_record(fbl, G, g, b, xt, device, peaks, iters=4):
     e1.record(stream)
     torch.cuda.synchronize(device)
     ms = e0.elapsed_time(e1) / reps
-    byt = float(n) * (24 + 72 * fgp + 20)
+    byt = float(n) * (12 + 40 * fgp + 20)
     gbs = byt / (ms * 1e-3) / 1e9
     tv_x = fbl.tv_norm(v)
     del q, xo
@@ -862,7 +861,7 @@ def run_tv_only(args):
     e1.record(stream)
     torch.cuda.synchronize(device)
     ms = e0.elapsed_time(e1) / reps
-    byt = float(g.n_vox) * (24 + 72 * fgp + 20)
+    byt = float(g.n_vox) * (12 + 40 * fgp + 20)
     return {"workload": args.workload, "prox_tv": {"voxels": g.n_vox, "fgp_iterations": fgp, "ms": ms,
                                                   "achieved_gbs": byt / (ms * 1e-3) / 1e9}}
 
@@ -935,7 +934,7 @@ def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
         "roofline_k1": alu_roofline("k1_project, residual (Step 2b, eq. (2.5))", K1_OPS_PER_SAMPLE,
                                     samples, k1_ms / max(k1_n, 1), g.n_vox * 4 + N_t * g.nu * g.nv * 4, clk,
                                     peaks),
-        "roofline_k2": alu_roofline("k2_backproject, gradient (Step 2b, eq. (2.5))", K2_OPS_PER_SAMPLE,
+        "roofline_k2": alu_roofline("k2_strips, gradient (Step 2b, eq. (2.5))", K2_OPS_PER_SAMPLE,
                                     samples, k2_ms / max(k2_n, 1),
                                     N_t * g.nu * (g.nv + 16) * 4 + g.n_vox * 4, clk, peaks,
                                     voxel_views_per_launch=float(N_t) * g.n_vox),
@@ -946,6 +945,12 @@ def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
         "kernels": {name: {"ms": round(v[0], 3), "launches": v[1]} for name, v in prof.items()},
         "clocks": clk,
     }
+
+
+def strip_launches(g):
+    """Launches of the strip backprojector over all views: one per 512 MiB of
+    weighted residual rows (nv + 16 floats per view and column)."""
+    return -(-(g.n_views * g.nu * (g.nv + 16) * 4) // (512 << 20))
 
 
 def sweep_units(g):
@@ -1017,7 +1022,7 @@ def run_kernels_only(args):
     the contract line): the workload's data (ceil(n_views/90) store-mode
     projector launches), then --steps trial-objective projections of one
     mini-batch (residual_norm: k_pack, k1_project, k_reduce) and --steps
-    backprojections of it (k_weight, k2_backproject, k_zi_to_natural), in the
+    backprojections of it (k_weight, k2_strips, k_zi_to_natural), in the
     launch configuration --launch (else the autotuner's, whose timing
     launches come first).  Prints the CUDA-event time of each."""
     import torch
@@ -1119,11 +1124,11 @@ def run_ours(args, rank, world, local_rank):
              "gsamples_in_volume_forward": in_vol / (fwd_ms * 1e-3) / 1e9,
              "units": "forward: n_views*nu*nv*N ray samples (nominal; in-volume ones beside); "
                       "back: n_views*N^3 voxel-views"}
-    # dominant kernel of the step: the backprojection of all views (one K2 launch;
-    # the call's events also hold its short weighting and reordering kernels)
+    # dominant kernel of the step: the backprojection of all views (K2, one launch
+    # per 512 MiB of rows; the call's events also hold its short weighting and reordering kernels)
     bp_bytes = g.n_views * g.nu * (g.nv + 16) * 4 + g.n_vox * 4
-    k2 = alu_roofline("k2_backproject over all %d views (one launch; the timed call also holds "
-                      "k_weight and k_zi_to_natural)" % g.n_views, K2_OPS_PER_SAMPLE, in_vol, bp_ms,
+    k2 = alu_roofline("k2_strips over all %d views (%d launches; the timed call also holds "
+                      "k_weight and k_zi_to_natural)" % (g.n_views, strip_launches(g)), K2_OPS_PER_SAMPLE, in_vol, bp_ms,
                       bp_bytes, clk, peaks, voxel_views_per_launch=bp_u)
     k1 = alu_roofline("k1_project, store mode, all %d views (one launch; the timed call also "
                       "holds k_pack)" % g.n_views, K1_OPS_PER_SAMPLE, in_vol, fwd_ms,
@@ -1140,9 +1145,9 @@ def run_ours(args, rank, world, local_rank):
                             % (g.n_vox * 4 / 1e6, g.n_views * g.nu * g.nv * 4 / 1e6),
                       "parallelism": "replicas" if world > 1 else "single GPU"},
            "full_sweep": sweep, "roofline": dominant, "roofline_other": other,
-           "gpu_launches": 5 * args.steps,
-           "gpu_launches_note": "per step: k_pack + k1_project (project call), k_weight + k2_backproject "
-                                "+ k_zi_to_natural (backproject call)",
+           "gpu_launches": (4 + strip_launches(g)) * args.steps,
+           "gpu_launches_note": "per step: k_pack + k1_project (project call), k_weight + k2_strips "
+                                "(%d launches) + k_zi_to_natural (backproject call)" % strip_launches(g),
            "clocks": clk, "autotune": tune, "peak_source": peak_src}
     del y, gr
 
