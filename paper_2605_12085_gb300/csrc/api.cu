@@ -2142,6 +2142,7 @@ fbl_status batch_iterate(fbl_batch *bt, const void *const *b, const char *b_dev,
         cfg.n_theta = d.n_views;
     }
     for (int ph = 0; ph < 3; ++ph) hh->total[ph] = first[ph];
+    hh->may_stop = batch_may_stop(bt->cols, first[0]) ? 1 : 0;
     hh->strip_tiles = bt->strip_vols < n ? hv[bt->strip_vols].first[1] : first[1];
     auto fail_all = [&](fbl_status r) {
         for (int v = 0; v < n; ++v) restore(v);

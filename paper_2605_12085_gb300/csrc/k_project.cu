@@ -710,8 +710,9 @@ __global__ void __launch_bounds__(32 * COLS, 48 / COLS) kb_project(const BatchHd
             sa.b_views = bv.b_views;
             sa.out = bv.rt;
             sa.partials = bv.partials;
-            sa.stop = MODE == PROJ_NORM ? bv.sc + 6 : nullptr;
-            if (MODE == PROJ_NORM) s_done = __ldcg(bv.sc + 6) > __ldcg(bv.sc + 7);
+            const bool stop = MODE == PROJ_NORM && hdr->may_stop;
+            sa.stop = stop ? bv.sc + 6 : nullptr;
+            s_done = stop && __ldcg(bv.sc + 6) > __ldcg(bv.sc + 7);
         }
         __syncthreads();
         const ProjArgs &a = sa;
@@ -870,18 +871,20 @@ int project_num_partials(const DevGeom &g, int n_sel) {
 }
 
 // Blocks of k1_project that are resident at once.
-static int first_wave(const DevGeom &g) {
+static int first_wave(int cols) {
     static const int sms = [] {
         int dev = 0, n = 0;
         cudaGetDevice(&dev);
         return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
     }();
-    return sms * (48 / (g.k1_cols == 4 ? 4 : 8));
+    return sms * (48 / (cols == 4 ? 4 : 8));
 }
 
 bool project_may_stop(const DevGeom &g, int n_sel) {
-    return g.k1_split != 2 && project_num_partials(g, n_sel) > first_wave(g);
+    return g.k1_split != 2 && project_num_partials(g, n_sel) > first_wave(g.k1_cols);
 }
+
+bool batch_may_stop(int cols, int64_t tiles) { return tiles > (int64_t)BATCH_STOP_WAVES * first_wave(cols); }
 
 cudaError_t launch_project(int mode, const DevGeom &g, const void *vol, ZLayout L, int x_dtype,
                            const int32_t *views, int n_sel, const void *b, int b_dtype,
@@ -901,7 +904,7 @@ cudaError_t launch_project(int mode, const DevGeom &g, const void *vol, ZLayout 
     a.out = out;
     a.partials = partials;
     a.stop = stop;
-    a.first = first_wave(g);
+    a.first = first_wave(g.k1_cols);
     if (n_partials) *n_partials = project_num_partials(g, n_sel);
     switch (x_dtype) {
         case FBL_BF16: return launch_bdt<__nv_bfloat16>(mode, b_dtype, out_dtype, a, n_sel, st);

@@ -265,9 +265,9 @@ __global__ void __launch_bounds__(R_NT) k_reduce_trial(const double *__restrict_
 
 // One block per (volume, component): the same fixed order as k_reduce over the
 // volume's tiles of phase ph (stride = its tile count).  The three sums of a trial
-// (ph 2) end with the trial's limit, as k_reduce_trial.
-__global__ void __launch_bounds__(R_NT) kb_reduce(const BatchVol *vols, int ph, int ncomp, int slot,
-                                                  int searching_only) {
+// (ph 2) end with the trial's limit, as k_reduce_trial, where blocks may leave.
+__global__ void __launch_bounds__(R_NT) kb_reduce(const BatchHdr *hdr, const BatchVol *vols, int ph, int ncomp,
+                                                  int slot, int searching_only) {
     const int v = blockIdx.x / ncomp, c = blockIdx.x % ncomp;
     const BatchVol &bv = vols[v];
     if (searching_only && !batch_searching(*bv.ls)) return;  // block-uniform
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(R_NT) kb_reduce(const BatchVol *vols, int ph, 
     const double s = block_reduce_fixed(bv.partials + (size_t)c * n, n);
     if (threadIdx.x != 0) return;
     bv.sc[slot + c] = s;
-    if (ph != 2) return;
+    if (ph != 2 || !hdr->may_stop) return;
     LSState &ls = *bv.ls;
     __threadfence();
     if (atomicAdd(&ls.ticket, 1) != 2) return;
@@ -423,8 +423,7 @@ cudaError_t launch_norms(const void *x, const void *xr, int dtype, int64_t n, do
 
 cudaError_t launch_batch_reduce(const BatchHdr *hdr, BatchVol *vols, int n_vol, int ph, int ncomp,
                                 int slot, int searching_only, cudaStream_t st) {
-    (void)hdr;
-    kb_reduce<<<n_vol * ncomp, R_NT, 0, st>>>(vols, ph, ncomp, slot, searching_only);
+    kb_reduce<<<n_vol * ncomp, R_NT, 0, st>>>(hdr, vols, ph, ncomp, slot, searching_only);
     return cudaGetLastError();
 }
 

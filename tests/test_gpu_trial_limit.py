@@ -71,3 +71,25 @@ def test_last_trial_of_a_failed_search_is_complete(graph):
     last = _trials(fbl, G, x0, b, S.last_batch(), p, 3)[-1]
     assert abs(st["f_xbar"] - last[1]) <= 1e-5 * last[1]
     assert abs(st["margin"] - (last[2] - last[1])) <= 1e-5 * last[1]
+
+
+@pytest.mark.parametrize("cols", [4, 8])
+def test_a_batch_large_enough_to_stop_its_trials_early(cols):
+    """Four volumes: more than eight waves of blocks, the batch's line for the limit
+    (a batch of one, above, lies below it)."""
+    import paper_2605_12085_gb300 as fbl
+    G, xt, b = _problem(fbl)
+    Gs = [G] + [fbl.geometry_create(G16) for _ in range(3)]
+    for q in Gs:
+        fbl.geometry_set_launch(q, cols, 1, 28)
+    ps = [fbl.params_default(N0=16, alpha0=1.0, mu=0.2, seed=9 + v) for v in range(4)]
+    S = fbl.fblisa_batch_create(Gs, ps)
+    xs = [(0.7 + 0.05 * v) * xt for v in range(4)]
+    for _ in range(2):
+        x0 = [x.clone() for x in xs]
+        for v, st in enumerate(S.step(xs, [b] * 4)):
+            tr = _trials(fbl, G, x0[v], b, S.last_batch(v), ps[v], st["backtracks"] + 1)
+            assert st["backtracks"] >= 3
+            assert all(f > rhs for _, f, rhs in tr[:-1]) and tr[-1][1] <= tr[-1][2]
+            assert abs(st["f_xbar"] - tr[-1][1]) <= 1e-5 * tr[-1][1]
+            assert rel_l2(host(xs[v]), host(tr[-1][0])) <= 1e-5
