@@ -193,8 +193,9 @@ FBL_API fbl_status geometry_autotune(fbl_geometry *g, int32_t x_dtype, int32_t n
  * backprojector's work per warp: 2 or 4 (24 the same) = one voxel column, with
  * that many consecutive voxels per lane; 8, 16 and 28 = strips of 8 voxel
  * columns, 6 voxels per lane for 16, else 4 or 8, whichever fills nz with less
- * work (28 and 8 are the same); a new geometry starts with 4 / 0 and a k2_vpl by
- * its volume's size; FBL_E_INVAL otherwise.  The batched solver runs k1_split 2
+ * work (28 and 8 are the same), and where some detector rows are more than 2
+ * voxels apart in the volume the same as 4; a new geometry starts with 4 / 0 and a
+ * k2_vpl by its volume's size; FBL_E_INVAL otherwise.  The batched solver runs k1_split 2
  * volumes with the loads-ahead loop. */
 FBL_API fbl_status geometry_set_launch(fbl_geometry *g, int32_t k1_cols, int32_t k1_split,
                                        int32_t k2_vpl);

@@ -256,7 +256,7 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
     std::vector<FxCol> colF(ncol);
     auto fx = [](double v) { return (long long)std::llround(v * FX_ONE); };
     std::vector<float2> trig(d.n_views);
-    double hw = 0.0, max_inv = 0.0;
+    double hw = 0.0, max_inv = 0.0, max_step = 0.0;
     for (int v = 0; v < d.n_views; ++v) {
         const double th = view_angle(d, g->angles, v);
         const double c = std::cos(th), sn = std::sin(th);
@@ -312,6 +312,7 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
                 for (double m : {mlo, mhi}) {
                     const double Zc = zc0 + m * zc1;
                     if (Zc > 0) max_inv = std::max(max_inv, 1.0 / (d.dv * Zc));
+                    max_step = std::max(max_step, d.dv * Zc);
                 }
         }
         // columns per voxel in-plane (the candidate window K2 searches): the
@@ -357,7 +358,8 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
     // 512^3 5.13; with 8 columns and loads one sample ahead 15.7, 0.357, 5.38)
     dg.k1_cols = 4;
     dg.k1_split = 0;
-    dg.k2_vpl = backproject_default_config(d.nx, d.ny, d.nz);
+    dg.wide_rows = max_step > STRIP_MAX_STEP ? 1 : 0;
+    dg.k2_vpl = backproject_default_config(dg);
     // detector rows with a crossing in (k - 1, k + 1) on one column: at most
     // floor(2 max_inv) + 1
     dg.ntap = (int)std::floor(2.0 * max_inv * 1.0001 + 0.002) + 1;
@@ -2268,9 +2270,9 @@ extern "C" fbl_status fblisa_batch_create(const fbl_geometry *const *geoms, cons
     }
     bt->order.resize(n_vol);
     for (int v = 0; v < n_vol; ++v) bt->order[v] = v;
-    for (int v = 0; v < n_vol; ++v) bt->strip_vols += k2_is_strips(geoms[v]->dg.k2_vpl) ? 1 : 0;
+    for (int v = 0; v < n_vol; ++v) bt->strip_vols += k2_is_strips(geoms[v]->dg) ? 1 : 0;
     std::stable_sort(bt->order.begin(), bt->order.end(), [&](int a, int c) {
-        const bool sa = k2_is_strips(geoms[a]->dg.k2_vpl), sc = k2_is_strips(geoms[c]->dg.k2_vpl);
+        const bool sa = k2_is_strips(geoms[a]->dg), sc = k2_is_strips(geoms[c]->dg);
         if (sa != sc) return sa;
         const fbl_geometry_desc &da = geoms[a]->desc, &dc = geoms[c]->desc;
         return (int64_t)da.nx * da.ny * da.nz > (int64_t)dc.nx * dc.ny * dc.nz;

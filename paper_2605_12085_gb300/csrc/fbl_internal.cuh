@@ -129,6 +129,7 @@ struct DevGeom {
     float sod, sdd, inv_du;
     float hwu;                   // half width, in columns, of a voxel's column footprint
     int ntap;                    // detector rows that can touch one voxel in one column
+    int wide_rows;               // some rows cross the volume more than STRIP_MAX_STEP voxels apart
     // launch configuration (by the autotuner; defaults 4 / 0 / by the volume's size)
     int k1_cols;                 // projector: detector columns per block (4 or 8)
     int k1_split;                // projector plane loop: 0 plain, 1 loads one sample ahead, 2 TMA-staged bricks
@@ -191,7 +192,7 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
                                double *g2_partials = nullptr);
 int backproject_num_partials(const DevGeom &g);
 // The k2_vpl a new geometry starts with.
-int backproject_default_config(int nx, int ny, int nz);
+int backproject_default_config(const DevGeom &g);
 
 struct BpArgs {
     DevGeom g;
@@ -208,7 +209,17 @@ struct BpArgs {
 // about ZP + 1.2 (8, 6 and 4 voxels per lane measured 0.90, 1.01 and 1.02 ps per
 // voxel and view where nz is a multiple of the span).
 constexpr int STRIP_EDGE = 8;
-__host__ __device__ __forceinline__ bool k2_is_strips(int k2_vpl) { return k2_vpl == 8 || k2_vpl == 16 || k2_vpl == 28; }
+// Strips hold a voxel's position as a fraction of a detector row to 23 bits, and
+// form the rows per voxel from a remainder of 32 bits: the error of their weights
+// grows with the voxels per row, and past 8 of them the remainder no longer fits.
+// Geometries with rows further apart than this run in columns, which hold the
+// position in voxels.  (Weights restated on the CPU against exact ones, rms over
+// 256 voxels: columns 1.7e-7 at every spacing, strips 1.3e-7 at 1 voxel, 1.8e-7 at
+// 1.2, 2.7e-7 at 2, 5e-7 at 4, 1e-6 at 8, 8e-5 at 12, 9e-4 at 110.)
+constexpr double STRIP_MAX_STEP = 2.0;
+__host__ __device__ __forceinline__ bool k2_is_strips(const DevGeom &g) {
+    return !g.wide_rows && (g.k2_vpl == 8 || g.k2_vpl == 16 || g.k2_vpl == 28);
+}
 __host__ __device__ __forceinline__ float strip_cost(int nz, int zp) {
     return (float)((nz + 32 * zp - 1) / (32 * zp)) * ((float)zp + 1.2f);
 }

@@ -7,8 +7,9 @@
 // y-planes), with weight wb * wz: wb from the in-plane crossing q_b(m) of its
 // detector column, wz from the vertical crossing q_z(m) of its row.
 //
-// Two forms.  Volumes large enough to fill the GPU run in strips (k_strips.cu).
-// Smaller ones run here, one voxel column per warp: many more and shorter warps
+// Two forms.  Volumes large enough to fill the GPU run in strips (k_strips.cu) where
+// the detector rows are at most STRIP_MAX_STEP voxels apart in them.
+// The others run here, one voxel column per warp: many more and shorter warps
 // (64^3, 10 views: 23.9 against 36 us).  A batch runs each volume in its own
 // geometry's form, so that its results are the single-volume solver's, although
 // a batch of small volumes fills the GPU and strips would be a little faster there
@@ -42,7 +43,8 @@ constexpr int K2_LANES = 32;
 
 // Launch configuration of the backprojector: k2_vpl 2 and 4 (24 the same) are
 // one voxel column per warp with that many consecutive voxels per lane; 8 and 28
-// are strips with 4 or 8 voxels per lane, 16 strips with 6.
+// are strips with 4 or 8 voxels per lane, 16 strips with 6 (all three run as 4
+// where the geometry's rows are too far apart for strips).
 __host__ __device__ __forceinline__ int k2_vpl_of(const DevGeom &g) { return g.k2_vpl == 2 ? 2 : 4; }
 constexpr int K2_WARPS = 8;   // consecutive i per block
 
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) kb_backproject(const Ba
 }  // namespace
 
 static dim3 k2_grid(const DevGeom &g) {
-    if (k2_is_strips(g.k2_vpl)) {
+    if (k2_is_strips(g)) {
         const unsigned span = 32 * strip_zp(g.k2_vpl, g.nz);
         return dim3((g.nx + STRIP_EDGE - 1) / STRIP_EDGE, (g.ny + STRIP_EDGE - 1) / STRIP_EDGE, (g.nz + span - 1) / span);
     }
@@ -336,12 +338,14 @@ int backproject_num_partials(const DevGeom &g) {
     return (int)(gr.x * gr.y * gr.z);
 }
 
-int backproject_default_config(int nx, int ny, int nz) {
+int backproject_default_config(const DevGeom &g) {
+    const int nx = g.nx, ny = g.ny, nz = g.nz;
     // fewer than 100 patches of 8 x 8 x 128 (80^3) leave SMs idle: one voxel column
     // per warp, 64 voxels high where that is enough (64^3, 10 views: 23.9 us with 2
     // voxels per lane, 28.0 with 4, 36 in strips; 96^3: 48.5 with 4, 37 in strips)
     const int64_t patches = (int64_t)((nx + 7) / 8) * ((ny + 7) / 8) * ((nz + 127) / 128);
     if (patches <= 100) return nz <= 64 ? 2 : 4;
+    if (g.wide_rows) return 4;
     return strip_cost(nz, 6) < strip_cost(nz, strip_zp(28, nz)) ? 16 : 28;
 }
 
@@ -395,7 +399,7 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
     a.gzi = gzi;
     dim3 block(K2_LANES, K2_WARPS);
     const dim3 grid = k2_grid(g);
-    if (k2_is_strips(g.k2_vpl)) return launch_strips(a, grid, strip_zp(g.k2_vpl, g.nz), st);
+    if (k2_is_strips(g)) return launch_strips(a, grid, strip_zp(g.k2_vpl, g.nz), st);
     const int vpl = k2_vpl_of(g);
     switch (g.ntap) {  // rows per voxel and column, fixed per geometry (<= RT_PAD)
         case 1: launch_k2<1>(vpl, grid, block, st, a); break;

@@ -170,7 +170,8 @@ __device__ __forceinline__ bool k2_entry(const BpArgs &a, int fam, int m, int bs
     constexpr float k2m40 = 9.094947017729282e-13f;  // 2^-40
     const float step = fmaf((float)(int)(S >> 20), 1048576.f, (float)(int)(S & 0xfffff)) * k2m40;
     // rows per voxel in Q.32: an FP32 reciprocal X and one correction by its
-    // exact remainder 2^72 - S X (below 2^51, so exact modulo 2^64)
+    // exact remainder 2^72 - S X (below 2^51 for rows up to 8 voxels apart, so exact
+    // modulo 2^64 and its top bits in 32; geometries here have at most STRIP_MAX_STEP)
     const float x0 = __fdividef(1.f, step);
     const unsigned long long X = (unsigned long long)__float2uint_rz(x0 * 16777216.f) << 8;
     const int R = (int)((long long)(0ull - (unsigned long long)S * X) >> 20);
