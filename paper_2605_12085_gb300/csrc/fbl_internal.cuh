@@ -214,8 +214,8 @@ constexpr int STRIP_EDGE = 8;
 // grows with the voxels per row, and past 8 of them the remainder no longer fits.
 // Geometries with rows further apart than this run in columns, which hold the
 // position in voxels.  (Weights restated on the CPU against exact ones, rms over
-// 256 voxels: columns 1.7e-7 at every spacing, strips 1.3e-7 at 1 voxel, 1.8e-7 at
-// 1.2, 2.7e-7 at 2, 5e-7 at 4, 1e-6 at 8, 8e-5 at 12, 9e-4 at 110.)
+// 256 voxels: columns 2.4e-7 at 1 voxel, 1.7e-7 from 1.5 on; strips 1.1e-7 at 1,
+// 1.3e-7 at 1.5, 1.5e-7 at 2, 2.1e-7 at 3, 3e-7 at 4, 8e-5 at 12, 9e-4 at 110.)
 constexpr double STRIP_MAX_STEP = 2.0;
 __host__ __device__ __forceinline__ bool k2_is_strips(const DevGeom &g) {
     return !g.wide_rows && (g.k2_vpl == 8 || g.k2_vpl == 16 || g.k2_vpl == 28);

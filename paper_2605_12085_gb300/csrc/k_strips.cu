@@ -187,7 +187,8 @@ __device__ __forceinline__ bool k2_entry(const BpArgs &a, int fam, int m, int bs
     const float zoff_f = g.cz - (float)(g.nv - 1) * 0.5f * step;
     const int r0 = (int)floorf(((float)kt - zoff_f) * x0);
     const long long d = ((long long)kt << FX_BITS) - zoff - (long long)r0 * S;  // about [0, S)
-    const long long t = ((long long)r0 << 32) + (((d >> 12) * inv) >> 28);
+    // (and half a unit of the 23 bits its fraction is cut to: rounded, not cut)
+    const long long t = ((long long)r0 << 32) + (((d >> 12) * inv) >> 28) + 256;
     // first rows of the strip's first and last voxel
     const int lo0 = fx32_floor(t) + off, lo1 = fx32_floor(t + (long long)(span - 1) * inv) + off;
     if (lo1 + taps <= 0 || lo0 >= g.nv) return false;  // only rows outside the detector

@@ -71,3 +71,22 @@ def test_batch_with_rows_far_apart_equals_single_solvers():
         for _ in range(3):
             S.step(x, b)
         assert np.array_equal(host(x), host(xb))
+
+
+@pytest.mark.parametrize("vpl", [16, 28])
+@pytest.mark.parametrize("spacing", [0.8, 1.2, 1.5, 1.7, 1.9])
+def test_strips_are_no_further_off_than_columns(spacing, vpl):
+    # one view at a time, so that the weights' error is not lost in the sums' rounding: strips
+    # hold a position to half of 2^-23 rows (up to 2 voxels), columns to a few 2^-24 voxels
+    import paper_2605_12085_gb300 as fbl
+    g = _geom(spacing, nx=16, ny=15, views=7)
+    G = fbl.geometry_create(g)
+    rng = np.random.default_rng(2)
+    err = {vpl: 0.0, 4: 0.0}
+    for v in range(g.n_views):
+        y = rng.standard_normal((1, g.nv, g.nu)).astype(np.float32)
+        ref = oracle.backproject(g, y.astype(np.float64), [v])
+        for form in err:
+            fbl.geometry_set_launch(G, 8, 1, form)
+            err[form] += rel_l2(host(fbl.backproject(G, cuda(y), [v])), ref) ** 2
+    assert err[vpl] <= err[4]
