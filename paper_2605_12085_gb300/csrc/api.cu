@@ -516,6 +516,24 @@ fbl_status upload_views(const int32_t *views, int32_t n, AsyncBuf &buf, cudaStre
     return FBL_OK;
 }
 
+// The same with a word behind the list that is 0 (in the same copy, but for a
+// captured call, whose copy reads the caller's list when the graph runs).
+fbl_status upload_views_and_zero(const int32_t *views, int32_t n, AsyncBuf &buf, cudaStream_t st) {
+    CK(buf.alloc(((size_t)n + 1) * sizeof(int32_t), st), "view list");
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        std::vector<int32_t> list(views, views + n);
+        list.push_back(0);
+        CK(cudaMemcpyAsync(buf.p, list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st),
+           "view list copy");
+        return FBL_OK;
+    }
+    cudaGetLastError();
+    CK(cudaMemcpyAsync(buf.p, views, (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, st), "view list copy");
+    CK(cudaMemsetAsync((int32_t *)buf.p + n, 0, sizeof(int32_t), st), "view list copy");
+    return FBL_OK;
+}
+
 // Device pointer for a caller buffer: itself if on the device, else a staged copy.
 fbl_status device_input(const void *p, size_t bytes, AsyncBuf &stage, const void **dev,
                         cudaStream_t st) {
@@ -670,16 +688,20 @@ extern "C" fbl_status backproject(const fbl_geometry *g, const void *y, int32_t 
     if (n_sel == 0) {
         if (!accumulate) CK(cudaMemsetAsync(xd, 0, nvox * sizeof(float), s), "memset");
     } else {
-        if ((st = upload_views(views, n_sel, dviews, s))) return st;
+        // strips take rows in that a voxel does not reach, with weight 0: they have to
+        // know of infinities and NaN
+        const bool strips = k2_is_strips(g->dg);
+        if ((st = strips ? upload_views_and_zero(views, n_sel, dviews, s) : upload_views(views, n_sel, dviews, s))) return st;
+        int *nonfinite = strips ? (int *)dviews.p + n_sel : nullptr;
         const void *yd = nullptr;
         if ((st = device_input(y, ny_in * dtype_size(y_dtype), ys, &yd, s))) return st;
         const size_t rt_elems = (size_t)n_sel * d.nu * rt_pitch(d.nv);
         CK(rt.alloc(rt_elems * sizeof(float), s), "weighted sinogram");
-        CK(launch_weight(g->dg, yd, y_dtype, (const int32_t *)dviews.p, n_sel, (float *)rt.p, s),
+        CK(launch_weight(g->dg, yd, y_dtype, (const int32_t *)dviews.p, n_sel, (float *)rt.p, nonfinite, s),
            "weight kernel");
         CK(gz.alloc(nvox * sizeof(float), s), "gradient scratch");
         CK(launch_backproject(g->dg, (const float *)rt.p, (const int32_t *)dviews.p, n_sel, 1.0f,
-                              (float *)gz.p, s),
+                              (float *)gz.p, s, nullptr, nonfinite),
            "backproject kernel");
         CK(launch_zi_to_natural((const float *)gz.p, xd, d.nx, d.ny, d.nz, accumulate, s), "reorder");
     }

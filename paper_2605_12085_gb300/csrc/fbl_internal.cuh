@@ -181,15 +181,16 @@ constexpr int BATCH_STOP_WAVES = 8;
 bool batch_may_stop(int cols, int64_t tiles);
 
 // rt[s][iu][RT_PAD + iv] = W(ray) * y[s][iv][iu] (the row weight folded in for K2),
-// and the rows' zero pads.
+// and the rows' zero pads; *nonfinite (if not NULL) becomes 1 where an entry is
+// infinite or NaN.
 cudaError_t launch_weight(const DevGeom &g, const void *y, int y_dtype, const int32_t *views,
-                          int n_sel, float *rt, cudaStream_t st);
+                          int n_sel, float *rt, int *nonfinite, cudaStream_t st);
 
 // gzi[j][i][k] = scale * sum over listed views of the transpose taps of rt;
 // with g2_partials, also the per-block sums of gzi^2 (backproject_num_partials).
 cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t *views,
                                int n_sel, float scale, float *gzi, cudaStream_t st,
-                               double *g2_partials = nullptr);
+                               double *g2_partials = nullptr, const int *nonfinite = nullptr);
 int backproject_num_partials(const DevGeom &g);
 // The k2_vpl a new geometry starts with.
 int backproject_default_config(const DevGeom &g);
@@ -202,6 +203,7 @@ struct BpArgs {
     float scale;
     float *gzi;
     double *g2_partials;  // optional: per-block sum of the squared gradient
+    const int *nonfinite; // strips, optional: not 0 where rt holds infinities or NaN (launch_weight)
     int more, last;       // strips: add to gzi's sums; scale the sum (and form its squares)
 };
 // The backprojector in strips (k_strips.cu): blocks of STRIP_EDGE x STRIP_EDGE

@@ -388,9 +388,10 @@ cudaError_t launch_batch_backproject(const BatchHdr *hdr, BatchVol *vols, int nt
 
 cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t *views,
                                int n_sel, float scale, float *gzi, cudaStream_t st,
-                               double *g2_partials) {
+                               double *g2_partials, const int *nonfinite) {
     BpArgs a;
     a.g2_partials = g2_partials;
+    a.nonfinite = nonfinite;
     a.g = g;
     a.rt = rt;
     a.views = views;

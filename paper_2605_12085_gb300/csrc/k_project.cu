@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(32 * COLS, 48 / COLS) kb_project(const BatchHd
 // 32 x 32 shared tile (reads along iu, writes along iv).
 template <typename TY>
 __global__ void __launch_bounds__(256) k_weight(const DevGeom g, const TY *__restrict__ y,
-                                                const int32_t *views, float *__restrict__ rt) {
+                                                const int32_t *views, float *__restrict__ rt, int *nonfinite) {
     __shared__ float tile[32][33];
     const int s = blockIdx.z;
     const int iu0 = blockIdx.x * 32, iv0 = blockIdx.y * 32;
@@ -763,7 +763,9 @@ __global__ void __launch_bounds__(256) k_weight(const DevGeom g, const TY *__res
             const float4 cB = g.colB[(size_t)v * g.nu + iu];
             const float w = (float)(2 * iv - (g.nv - 1)) * (0.5f * g.dv);
             const float W = cB.x * sqrtf(fmaf(w, w, cB.y));
-            tile[ty + 8 * r][tx] = W * to_f32(y[((size_t)s * g.nv + iv) * g.nu + iu]);
+            const float t = W * to_f32(y[((size_t)s * g.nv + iv) * g.nu + iu]);
+            tile[ty + 8 * r][tx] = t;
+            if (nonfinite && !isfinite(t)) *nonfinite = 1;
         }
     }
     __syncthreads();
@@ -952,14 +954,14 @@ cudaError_t launch_batch_project(int mode, const BatchHdr *hdr, BatchVol *vols, 
 }
 
 cudaError_t launch_weight(const DevGeom &g, const void *y, int y_dtype, const int32_t *views,
-                          int n_sel, float *rt, cudaStream_t st) {
+                          int n_sel, float *rt, int *nonfinite, cudaStream_t st) {
     if (n_sel <= 0) return cudaSuccess;
     dim3 block(32, 8);
     dim3 grid((g.nu + 31) / 32, (g.nv + 31) / 32, n_sel);
     switch (y_dtype) {
-        case FBL_BF16: k_weight<<<grid, block, 0, st>>>(g, (const __nv_bfloat16 *)y, views, rt); break;
-        case FBL_F16: k_weight<<<grid, block, 0, st>>>(g, (const __half *)y, views, rt); break;
-        default: k_weight<<<grid, block, 0, st>>>(g, (const float *)y, views, rt); break;
+        case FBL_BF16: k_weight<<<grid, block, 0, st>>>(g, (const __nv_bfloat16 *)y, views, rt, nonfinite); break;
+        case FBL_F16: k_weight<<<grid, block, 0, st>>>(g, (const __half *)y, views, rt, nonfinite); break;
+        default: k_weight<<<grid, block, 0, st>>>(g, (const float *)y, views, rt, nonfinite); break;
     }
     return cudaGetLastError();
 }

@@ -155,6 +155,9 @@ template <int KIND> struct K2Taps {
 
 // The constants of column iu of batch slot s in plane m, for the strip of
 // voxels [bs, bs + edge) x [kb, kb + span); false if it does not reach the strip.
+// MASKED: some residual is infinite or NaN, every profile is of the kind that
+// leaves rows of weight 0 out.
+template <bool MASKED>
 __device__ __forceinline__ bool k2_entry(const BpArgs &a, int fam, int m, int bs, int edge, int kb, int span, int s,
                                          int v, int iu, K2Entry &e) {
     const DevGeom &g = a.g;
@@ -178,7 +181,7 @@ __device__ __forceinline__ bool k2_entry(const BpArgs &a, int fam, int m, int bs
     const long long inv = (long long)X + __float2int_rn((float)R * x0 * (1.f / 1048576.f));
     const int whole = (int)(inv >> 32);
     const unsigned invf = (unsigned)inv;
-    const int kind = whole == 0 ? K2_TWO : (whole == 1 ? (invf <= 0x80000000u ? K2_THREE : K2_FOUR) : K2_MANY);
+    const int kind = MASKED ? K2_MANY : whole == 0 ? K2_TWO : (whole == 1 ? (invf <= 0x80000000u ? K2_THREE : K2_FOUR) : K2_MANY);
     const int taps = kind == K2_MANY ? RT_PAD : kind + 2;
     const bool bracket = kind == K2_TWO || kind == K2_FOUR;
     const int off = kind == K2_TWO ? 0 : (kind == K2_FOUR ? -1 : 1);
@@ -238,7 +241,7 @@ __device__ __forceinline__ void k2_weights(F2 f1, float step, F2 (&w)[K2Taps<KIN
 // (row coordinate t).  The whole rows per voxel go into the row pointer (0 or
 // 1, known from the kind), the fraction times k into t with one 32 x 32 + 64
 // bit multiply-add.
-template <int KIND, int ZP>
+template <int KIND, int ZP, bool MASKED = false>
 __device__ __forceinline__ void k2_profile(float (&P)[ZP], const float *__restrict__ row, unsigned long long t,
                                            unsigned invf, int whole, float step, int nv) {
     constexpr int taps = K2Taps<KIND>::taps, off = K2Taps<KIND>::off;
@@ -265,9 +268,19 @@ __device__ __forceinline__ void k2_profile(float (&P)[ZP], const float *__restri
         F2 w[taps];
         k2_weights<KIND>(F2{frac1(ta), frac1(tb)}, step, w);
         const float *ra = rows(ta, q), *rb = rows(tb, q + 1);
-        F2 p = pk_mul(w[0], F2{__ldg(ra), __ldg(rb)});
+        F2 p{0.f, 0.f};
+        if constexpr (MASKED) {  // a row that does not reach the voxel may hold an infinity or NaN
 #pragma unroll
-        for (int j = 1; j < taps; ++j) p = pk_fma(w[j], F2{__ldg(ra + j), __ldg(rb + j)}, p);
+            for (int j = 0; j < taps; ++j) {
+                const float xa = __ldg(ra + j), xb = __ldg(rb + j);
+                if (w[j].x > 0.f) p.x = fmaf(w[j].x, xa, p.x);
+                if (w[j].y > 0.f) p.y = fmaf(w[j].y, xb, p.y);
+            }
+        } else {
+            p = pk_mul(w[0], F2{__ldg(ra), __ldg(rb)});
+#pragma unroll
+            for (int j = 1; j < taps; ++j) p = pk_fma(w[j], F2{__ldg(ra + j), __ldg(rb + j)}, p);
+        }
         P[q] = p.x;
         P[q + 1] = p.y;
     }
@@ -292,7 +305,7 @@ struct K2List {
 };
 
 // One entry: its profile P times 1 - w1 into A (the strip's voxel rel) and w1 into B (rel + 1).
-template <int ZP>
+template <int ZP, bool MASKED>
 __device__ __forceinline__ void k2_add(const K2Entry *e, int nv, float (&A)[ZP], float (&B)[ZP]) {
     const int4 wa = reinterpret_cast<const int4 *>(e)[0], wb = reinterpret_cast<const int4 *>(e)[1];
     const unsigned long long t = ((unsigned long long)(unsigned)wa.w << 32) | (unsigned)wa.z;
@@ -300,6 +313,12 @@ __device__ __forceinline__ void k2_add(const K2Entry *e, int nv, float (&A)[ZP],
     const unsigned invf = (unsigned)wb.x;
     const float step = __int_as_float(wb.y), w1 = __int_as_float(wb.z), w0 = 1.f - w1;
     float P[ZP];
+    if constexpr (MASKED) {  // (w1 may be 0 and P infinite or NaN)
+        k2_profile<K2_MANY | K2_CLAMP, ZP, true>(P, row, t, invf, wb.w >> 16, step, nv);
+        k2_axpy<ZP>(w0, P, A);
+        if (w1 != 0.f) k2_axpy<ZP>(w1, P, B);
+        return;
+    }
     const int kind = (wb.w >> 8) & 7;
     if (kind == K2_TWO) k2_profile<K2_TWO, ZP>(P, row, t, invf, 0, step, nv);
     else if (kind == K2_THREE) k2_profile<K2_THREE, ZP>(P, row, t, invf, 0, step, nv);
@@ -315,7 +334,7 @@ __device__ __forceinline__ void k2_add(const K2Entry *e, int nv, float (&A)[ZP],
 // The n listed profiles into the strip's voxels (voxel b at tensor-memory column
 // strip + b ZP): ordered by rel with warp votes, then summed voxel by voxel
 // in registers, each voxel's sum added to tensor memory once.
-template <int EDGE, int ZP>
+template <int EDGE, int ZP, bool MASKED>
 __device__ __forceinline__ void k2_sum(K2List &L, int n, int nv, unsigned strip) {
     const int lane = threadIdx.x & 31;
     constexpr int G = (K2_CAP + 31) / 32;
@@ -347,7 +366,7 @@ __device__ __forceinline__ void k2_sum(K2List &L, int n, int nv, unsigned strip)
         }
         const int end = L.end[b];
 #pragma unroll 1
-        for (; p < end; ++p) k2_add<ZP>(&L.e[L.order[p]], nv, A, B);
+        for (; p < end; ++p) k2_add<ZP, MASKED>(&L.e[L.order[p]], nv, A, B);
         if (b > 0) {
             float C[ZP];
             __syncwarp();
@@ -363,7 +382,7 @@ __device__ __forceinline__ void k2_sum(K2List &L, int n, int nv, unsigned strip)
 }
 
 // One warp's strip: the profiles of family fam from all batch slots.
-template <int EDGE, int ZP>
+template <int EDGE, int ZP, bool MASKED>
 __device__ __forceinline__ void k2_strip(const BpArgs &a, int fam, int m, int bs, int kb, K2List &L,
                                          unsigned strip) {
     const DevGeom &g = a.g;
@@ -409,19 +428,19 @@ __device__ __forceinline__ void k2_strip(const BpArgs &a, int fam, int m, int bs
             for (int r = 0; r < rounds; ++r) {
                 const int iu = l + (lane & 15) + 16 * r;
                 K2Entry e;
-                const bool on = iu <= h && k2_entry(a, fam, m, bs, EDGE, kb, 32 * ZP, s0 + src, vv, iu, e);
+                const bool on = iu <= h && k2_entry<MASKED>(a, fam, m, bs, EDGE, kb, 32 * ZP, s0 + src, vv, iu, e);
                 const unsigned mask = __ballot_sync(0xffffffffu, on);
                 if (on) L.e[n + __popc(mask & ((1u << lane) - 1u))] = e;
                 __syncwarp();
                 n += __popc(mask);
                 if (n > K2_CAP - 32) {
-                    k2_sum<EDGE, ZP>(L, n, g.nv, strip);
+                    k2_sum<EDGE, ZP, MASKED>(L, n, g.nv, strip);
                     n = 0;
                 }
             }
         }
     }
-    if (n > 0) k2_sum<EDGE, ZP>(L, n, g.nv, strip);
+    if (n > 0) k2_sum<EDGE, ZP, MASKED>(L, n, g.nv, strip);
 }
 
 // One block's patch: voxel columns [EDGE bx, ..) x [EDGE by, ..), z-span bz;
@@ -435,7 +454,7 @@ struct K2Smem {
     K2List lists[WARPS];
     unsigned tmem;
 };
-template <int EDGE, int ZP, int WARPS>
+template <int EDGE, int ZP, int WARPS, bool MASKED = false>
 __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int bx, int by, int bz, double *g2_partial) {
     const DevGeom &g = a.g;
     const int lane = threadIdx.x & 31, w0 = threadIdx.x >> 5;
@@ -452,7 +471,7 @@ __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int 
             __syncwarp();
 #pragma unroll 1
             for (int b = 0; b < EDGE; ++b) tm_st<ZP>(strip + b * ZP, C);
-            k2_strip<EDGE, ZP>(a, fam, (fam ? j0 : i0) + w, fam ? i0 : j0, kb, sm.lists[w0], strip);
+            k2_strip<EDGE, ZP, MASKED>(a, fam, (fam ? j0 : i0) + w, fam ? i0 : j0, kb, sm.lists[w0], strip);
             if (!fam && w == w0) __syncthreads();  // every y-plane's sums are in gzi
             __syncwarp();
             tm_wait_st();
@@ -487,18 +506,28 @@ __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int 
     }
 }
 
+// The patch with infinities or NaN among the residuals: a call of its own, so that
+// the usual path keeps its registers (the mask as a flag inside it: 406 -> 431 us for
+// 20 views at 256^3).
+template <int ZP>
+__device__ __noinline__ void k2_tile_masked(const BpArgs &a, K2Smem<STRIP_EDGE> &sm) {
+    k2_tile<STRIP_EDGE, ZP, STRIP_EDGE, true>(a, sm, blockIdx.x, blockIdx.y, blockIdx.z, nullptr);
+}
+
 // At most 64 registers (4 blocks per SM, 32 warps): 4.79 against 4.84 ms per
 // 40-view launch at 512^3 with 80 registers and 3 blocks, 1.14 against 1.20 ms at
 // 384^3 with 6 voxels per lane; the few spilled values lie outside the inner loops.
 template <int ZP>
-__global__ void __launch_bounds__(32 * STRIP_EDGE, 4) k2_strips(const BpArgs a) {
+__global__ void __launch_bounds__(32 * STRIP_EDGE, 4) k2_strips(const __grid_constant__ BpArgs a) {
     const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     __shared__ K2Smem<STRIP_EDGE> sm;
     constexpr int cols = tm_cols(STRIP_EDGE, STRIP_EDGE, ZP);
     if (threadIdx.x < 32) tm_alloc(&sm.tmem, cols);
     __syncthreads();
-    k2_tile<STRIP_EDGE, ZP, STRIP_EDGE>(a, sm, blockIdx.x, blockIdx.y, blockIdx.z,
-                                        a.g2_partials ? a.g2_partials + blk : nullptr);
+    if (a.nonfinite && __ldcg(a.nonfinite)) k2_tile_masked<ZP>(a, sm);
+    else
+        k2_tile<STRIP_EDGE, ZP, STRIP_EDGE>(a, sm, blockIdx.x, blockIdx.y, blockIdx.z,
+                                            a.g2_partials ? a.g2_partials + blk : nullptr);
     __syncthreads();
     if (threadIdx.x < 32) tm_free(sm.tmem, cols);
 }
@@ -534,6 +563,7 @@ __global__ void __launch_bounds__(32 * KBS_WARPS, KBS_BLOCKS) kb_strips(const Ba
             sa.scale = bv.scale;
             sa.gzi = bv.grad;
             sa.g2_partials = bv.partials;
+            sa.nonfinite = nullptr;  // (a solver's step fails where a residual is not finite)
             sa.more = 0;
             sa.last = 1;
         }
