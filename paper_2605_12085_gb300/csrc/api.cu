@@ -1464,9 +1464,9 @@ fbl_status solver_iterate(fbl_solver *s, const void *b, bool b_dev, fbl_step_sta
         gTd = s->h_sc[1];
         dd = s->h_sc[2];
         rho1 = s->h_sc[4];
-        f_x = 0.5 * scale * rho0;
-        f_xb = 0.5 * scale * rho1;
-        rhs = f_x + gTd + dd / (2.0 * alpha);
+        f_x = ls_objective(scale, rho0);
+        f_xb = ls_objective(scale, rho1);
+        rhs = ls_rhs(scale, rho0, gTd, dd, alpha);
         if (!std::isfinite(f_x) || !std::isfinite(f_xb) || !std::isfinite(rhs)) {
             restore();
             return fail(FBL_E_NONFINITE, "fblisa_step: non-finite objective or reduction at k=%lld",

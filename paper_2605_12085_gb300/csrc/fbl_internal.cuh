@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fbl_linesearch.h"
 #include "fblisa.h"
 
 namespace fbl {

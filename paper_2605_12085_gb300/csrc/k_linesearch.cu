@@ -2,9 +2,8 @@
 // for the graph-captured iteration: the prox kernel reads the trial step from
 // device memory, and after each trial a one-thread kernel evaluates the
 // sufficient-decrease test (2.3) in FP64 and sets the condition of the
-// graph's WHILE node.  The arithmetic is the host loop's, operation by
-// operation, with explicitly rounded FP64 intrinsics (no contraction into
-// FMA), so both modes take identical decisions.
+// graph's WHILE node.  The arithmetic is the host loop's (fbl_linesearch.h), so
+// both modes take identical decisions.
 #include <math.h>
 
 #include "fbl_internal.cuh"
@@ -145,10 +144,9 @@ __global__ void kb_ls_init(BatchHdr *hdr, BatchVol *vols, int n_vol) {
 __device__ __forceinline__ unsigned int ls_decide_one(LSState *ls, PropState *ps, const double *sc) {
     const double rho0 = sc[0], gTd = sc[1], dd = sc[2], rho1 = sc[4];
     const double alpha = ls->alpha;
-    const double half_scale = __dmul_rn(0.5, ls->scale);
-    const double f_x = __dmul_rn(half_scale, rho0);
-    const double f_xb = __dmul_rn(half_scale, rho1);
-    const double rhs = __dadd_rn(__dadd_rn(f_x, gTd), __ddiv_rn(dd, __dmul_rn(2.0, alpha)));
+    const double f_x = ls_objective(ls->scale, rho0);
+    const double f_xb = ls_objective(ls->scale, rho1);
+    const double rhs = ls_rhs(ls->scale, rho0, gTd, dd, alpha);
     ls->rho0 = rho0;
     ls->gTd = gTd;
     ls->dd = dd;

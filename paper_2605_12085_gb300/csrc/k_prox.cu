@@ -234,17 +234,16 @@ __global__ void __launch_bounds__(R_NT) k_reduce(const double *__restrict__ part
 
 // The limit of a trial's rho1 (see launch_reduce_trial).  The trial is rejected
 // when f_N(x_bar) > rhs, and f_N(x_bar) is a sum of squares: a partial sum above
-// the limit settles it.  The margin of 1e-9 covers the order of the FP64 sums
-// (at most 2^20 terms).  The objective is completed where a rejected trial's
+// the limit settles it.  The objective is completed where a rejected trial's
 // value is reported or checked: at the last trial, and where a square could
 // overflow FP32 (the bounds keep |A x_bar - b| below 1e18, so a trial that is
 // stopped early cannot hide a non-finite objective).
 __device__ __forceinline__ void trial_limit(double *sc, double alpha, double scale, bool last, float wmax) {
     const double rho0 = __ldcg(sc), gTd = __ldcg(sc + 1), dd = __ldcg(sc + 2), l1 = __ldcg(sc + 3);
-    const double half = 0.5 * scale, rhs = half * rho0 + gTd + dd / (2.0 * alpha);
+    const double rhs = ls_rhs(scale, rho0, gTd, dd, alpha);
     const bool bounded = rho0 < 1e24 && dd < 1e20 && l1 < 1e15 && wmax < 100.f && isfinite(rhs);
     sc[6] = 0.0;
-    sc[7] = bounded && !last ? fmax(rhs, 0.0) / half * (1.0 + 1e-9) : INFINITY;
+    sc[7] = bounded && !last ? ls_limit(scale, rhs) : INFINITY;
 }
 
 // k_reduce of the three sums of a trial; the last of its three blocks sets the
