@@ -453,6 +453,7 @@ template <int WARPS>
 struct K2Smem {
     K2List lists[WARPS];
     unsigned tmem;
+    float g2[STRIP_EDGE];  // a block of fewer warps than planes: each plane's sum of squares
 };
 template <int EDGE, int ZP, int WARPS, bool MASKED = false>
 __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int bx, int by, int bz, double *g2_partial) {
@@ -496,9 +497,24 @@ __device__ __forceinline__ void k2_tile(const BpArgs &a, K2Smem<WARPS> &sm, int 
                     }
                 }
             }
+            if (WARPS < EDGE && !fam) {
+                g2 = warp_sum_f32(g2);
+                if (lane == 0) sm.g2[w] = g2;
+                g2 = 0.f;
+            }
         }
     }
-    if (g2_partial) {
+    if (WARPS < EDGE) {
+        // the planes' sums in the order that a block of one plane per warp adds them in,
+        // so that a batch reports the single-volume solver's ||g||^2
+        __syncthreads();
+        if (g2_partial && threadIdx.x == 0) {
+            double o = 0.0;
+#pragma unroll 1
+            for (int w = 0; w < EDGE; ++w) o += (double)sm.g2[w];
+            *g2_partial = o;
+        }
+    } else if (g2_partial) {
         float vv[1] = {g2};
         double o[1];
         block_sum_f64<32 * WARPS, 1>(vv, o);
