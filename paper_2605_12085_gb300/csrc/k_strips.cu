@@ -548,10 +548,33 @@ __global__ void __launch_bounds__(32 * STRIP_EDGE, 4) k2_strips(const __grid_con
     if (threadIdx.x < 32) tm_free(sm.tmem, cols);
 }
 
+// Views a launch takes at most: 512 MiB of residual rows.  The blocks of a launch
+// walk its views in order but drift apart; over 1.7 GB of rows (720 views at 512^3)
+// the re-reads from DRAM cost more than adding into the gradient again (107 ms in one
+// launch, 91 in four), up to 0.5 GB they do not (720 views at 256^3: 12.3 ms in one
+// launch, 13.4 in five; 200 at 512^3: 24.7 and 24.8).
+constexpr size_t STRIP_BYTES = size_t(512) << 20;
+__host__ __device__ __forceinline__ int strip_parts(const DevGeom &g, int n_sel) {
+    const size_t bytes = (size_t)n_sel * g.nu * rt_pitch(g.nv) * sizeof(float);
+    const size_t parts = (bytes + STRIP_BYTES - 1) / STRIP_BYTES;
+    return (int)(parts < (size_t)n_sel ? parts : (size_t)n_sel);
+}
+// The rows and views of part p of n_sel.
+__host__ __device__ __forceinline__ void strip_part(BpArgs &a, const float *rt, const int32_t *views, int n_sel, int p,
+                                                    int parts) {
+    const int s0 = (int)((int64_t)n_sel * p / parts), s1 = (int)((int64_t)n_sel * (p + 1) / parts);
+    a.rt = rt + (size_t)s0 * a.g.nu * rt_pitch(a.g.nv);
+    a.views = views + s0;
+    a.n_sel = s1 - s0;
+    a.more = p > 0;
+    a.last = p + 1 == parts;
+}
+
 // Persistent batched strips: the patches of the volumes that run in strips (the
 // first `total` tiles of the phase), taken from an atomic counter.  Each volume
-// keeps its own voxels per lane (a block-uniform switch), so its sums are those
-// of its single-volume launch; a block is 4 warps, which take two planes each.
+// keeps its own voxels per lane (a block-uniform switch) and the parts that its
+// views run in (launch_strips), so its sums are those of its single-volume
+// launches; a block is 4 warps, which take two planes each.
 constexpr int KBS_WARPS = 4, KBS_BLOCKS = 5;
 static_assert(KBS_BLOCKS * tm_cols(KBS_WARPS, STRIP_EDGE, 8) <= 512, "tensor memory of an SM");
 __global__ void __launch_bounds__(32 * KBS_WARPS, KBS_BLOCKS) kb_strips(const BatchHdr *hdr, const BatchVol *vols, int *ctr) {
@@ -573,26 +596,27 @@ __global__ void __launch_bounds__(32 * KBS_WARPS, KBS_BLOCKS) kb_strips(const Ba
         // the volume's arguments, staged in shared memory for the whole block
         stage_words(&sa.g, &bv.g, sizeof(DevGeom), tid, 32 * KBS_WARPS);
         if (tid == 0) {
-            sa.rt = bv.rt;
-            sa.views = bv.views;
-            sa.n_sel = bv.N_t;
             sa.scale = bv.scale;
             sa.gzi = bv.grad;
             sa.g2_partials = bv.partials;
             sa.nonfinite = nullptr;  // (a solver's step fails where a residual is not finite)
-            sa.more = 0;
-            sa.last = 1;
         }
-        __syncthreads();
         const BpArgs &a = sa;
         const int local = t - bv.first[1];
         const int gx = (bv.g.nx + STRIP_EDGE - 1) / STRIP_EDGE, gy = (bv.g.ny + STRIP_EDGE - 1) / STRIP_EDGE;
         const int bx = local % gx, rest = local / gx, by = rest % gy, bz = rest / gy;
-        double *part = bv.partials + local;
-        switch (strip_zp(bv.g.k2_vpl, bv.g.nz)) {
-            case 4: k2_tile<STRIP_EDGE, 4, KBS_WARPS>(a, sm, bx, by, bz, part); break;
-            case 6: k2_tile<STRIP_EDGE, 6, KBS_WARPS>(a, sm, bx, by, bz, part); break;
-            default: k2_tile<STRIP_EDGE, 8, KBS_WARPS>(a, sm, bx, by, bz, part); break;
+        const int parts = strip_parts(bv.g, bv.N_t);
+#pragma unroll 1
+        for (int p = 0; p < parts; ++p) {
+            if (p > 0) __syncthreads();  // the last part's arguments and sums
+            if (tid == 0) strip_part(sa, bv.rt, bv.views, bv.N_t, p, parts);
+            __syncthreads();
+            double *part = a.last ? bv.partials + local : nullptr;
+            switch (strip_zp(bv.g.k2_vpl, bv.g.nz)) {
+                case 4: k2_tile<STRIP_EDGE, 4, KBS_WARPS>(a, sm, bx, by, bz, part); break;
+                case 6: k2_tile<STRIP_EDGE, 6, KBS_WARPS>(a, sm, bx, by, bz, part); break;
+                default: k2_tile<STRIP_EDGE, 8, KBS_WARPS>(a, sm, bx, by, bz, part); break;
+            }
         }
     }
     __syncthreads();
@@ -618,25 +642,12 @@ cudaError_t launch_batch_strips(const BatchHdr *hdr, BatchVol *vols, int *ctr, c
     return cudaGetLastError();
 }
 
-// Views a launch takes at most: 512 MiB of residual rows.  The blocks of a launch
-// walk its views in order but drift apart; over 1.7 GB of rows (720 views at 512^3)
-// the re-reads from DRAM cost more than adding into the gradient again (107 ms in one
-// launch, 91 in four), up to 0.5 GB they do not (720 views at 256^3: 12.3 ms in one
-// launch, 13.4 in five; 200 at 512^3: 24.7 and 24.8).
-constexpr size_t STRIP_BYTES = size_t(512) << 20;
-
 cudaError_t launch_strips(const BpArgs &a, dim3 grid, int zp, cudaStream_t st) {
     auto k = zp == 4 ? k2_strips<4> : zp == 6 ? k2_strips<6> : k2_strips<8>;
-    const size_t bytes = (size_t)a.n_sel * a.g.nu * rt_pitch(a.g.nv) * sizeof(float);
-    const int parts = (int)std::min((bytes + STRIP_BYTES - 1) / STRIP_BYTES, (size_t)std::max(1, a.n_sel));
+    const int parts = strip_parts(a.g, a.n_sel);
     for (int p = 0; p < parts; ++p) {
-        const int s0 = (int)((int64_t)a.n_sel * p / parts), s1 = (int)((int64_t)a.n_sel * (p + 1) / parts);
         BpArgs b = a;
-        b.rt = a.rt + (size_t)s0 * a.g.nu * rt_pitch(a.g.nv);
-        b.views = a.views + s0;
-        b.n_sel = s1 - s0;
-        b.more = p > 0;
-        b.last = p + 1 == parts;
+        strip_part(b, a.rt, a.views, a.n_sel, p, parts);
         if (!b.last) b.g2_partials = nullptr;
         k<<<grid, 32 * STRIP_EDGE, 0, st>>>(b);
     }
