@@ -281,9 +281,12 @@ __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) k2_backproject(const Bp
 // Persistent batched backprojector: the blocks of k2_backproject of every volume
 // that does not run in strips (the tiles from hdr->strip_tiles on), taken from an
 // atomic counter.  Each volume keeps its own voxels per lane (its geometry's
-// k2_vpl, a warp-uniform switch).
+// k2_vpl, a warp-uniform switch).  At most 64 registers (4 blocks per SM): with the
+// single-volume kernel's 48 it spills, 12 iterations of 4 volumes of 20^3..41^3 took
+// 2.42 instead of 2.35 ms (4 voxels per lane; BF16), 16 of 96^3..320^3 in columns 42.2
+// instead of 41.6 ms per iteration (learned first step).
 template <int NTAP>
-__global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) kb_backproject(const BatchHdr *hdr,
+__global__ void __launch_bounds__(K2_LANES *K2_WARPS, 4) kb_backproject(const BatchHdr *hdr,
                                                                         const BatchVol *vols, int *ctr) {
     __shared__ int s_tile;
     __shared__ BpArgs sa;
