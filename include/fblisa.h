@@ -170,7 +170,8 @@ FBL_API void geometry_destroy(fbl_geometry *g);
 /* Launch configurations tried by the autotuner and their measured times. */
 typedef struct {
     float k1_ms[5];     /* projector, (cols, k1_split) = (8,1), (8,0), (4,1), (4,0), (8,2) */
-    float k2_ms[6];     /* backprojector, k2_vpl = 4, 2, 8, 16, 24, 28 (geometry_set_launch) */
+    float k2_ms[6];     /* backprojector, k2_vpl = 4, 2, 8, 16, 24, 28 (geometry_set_launch);
+                           those that are the same launch are timed once and share the time */
     int32_t k1_cols, k1_split, k2_vpl;  /* the chosen configuration */
 } fbl_tune_report;
 

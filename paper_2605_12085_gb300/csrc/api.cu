@@ -1647,9 +1647,24 @@ fbl_status autotune_devgeom(const fbl_geometry *g, DevGeom &dg, int x_dtype, int
     }
     best = 1e30f;
     qi = 0;
-    for (int vpl : {4, 2, 8, 16, 24, 28}) {
+    float k2_ms[6] = {};
+    constexpr int k2_cfg[6] = {4, 2, 8, 16, 24, 28};
+    for (int vpl : k2_cfg) {
         DevGeom t = dg;
         t.k2_vpl = vpl;
+        // a configuration that runs as an earlier one has its time
+        int same = -1;
+        for (int q = 0; q < qi && same < 0; ++q) {
+            DevGeom o = dg;
+            o.k2_vpl = k2_cfg[q];
+            if (backproject_same_launch(t, o)) same = q;
+        }
+        if (same >= 0) {
+            k2_ms[qi] = k2_ms[same];
+            if (rep) rep->k2_ms[qi] = k2_ms[qi];
+            ++qi;
+            continue;
+        }
         float ms = 0.f;
         cudaError_t e = time_it(
             [&] {
@@ -1662,7 +1677,8 @@ fbl_status autotune_devgeom(const fbl_geometry *g, DevGeom &dg, int x_dtype, int
             cudaEventDestroy(e1);
             return cuda_fail(e, "autotune backprojector");
         }
-        if (rep && qi < 6) rep->k2_ms[qi] = ms;
+        k2_ms[qi] = ms;
+        if (rep) rep->k2_ms[qi] = ms;
         ++qi;
         if (ms < best) {
             best = ms;

@@ -195,6 +195,8 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
 int backproject_num_partials(const DevGeom &g);
 // The k2_vpl a new geometry starts with.
 int backproject_default_config(const DevGeom &g);
+// Whether two configurations of a geometry are the same launch.
+bool backproject_same_launch(const DevGeom &a, const DevGeom &b);
 
 struct BpArgs {
     DevGeom g;

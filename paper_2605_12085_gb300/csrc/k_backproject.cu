@@ -352,6 +352,11 @@ int backproject_default_config(const DevGeom &g) {
     return strip_cost(nz, 6) < strip_cost(nz, strip_zp(28, nz)) ? 16 : 28;
 }
 
+bool backproject_same_launch(const DevGeom &a, const DevGeom &b) {
+    if (k2_is_strips(a) != k2_is_strips(b)) return false;
+    return k2_is_strips(a) ? strip_zp(a.k2_vpl, a.nz) == strip_zp(b.k2_vpl, b.nz) : k2_vpl_of(a) == k2_vpl_of(b);
+}
+
 template <int NT>
 static void launch_k2(int vpl, dim3 grid, dim3 block, cudaStream_t st, const BpArgs &a) {
     if (vpl == 2) k2_backproject<NT, 2><<<grid, block, 0, st>>>(a);
