@@ -73,8 +73,11 @@ __global__ void __launch_bounds__(TV_NT) k_tv_primal(const float *__restrict__ b
 // and finishes the dual of the plane below, whose neighbours' y are known now.
 // HBM-bound: the halo's second reads come from L2 (TS_W = 30 of 32 lanes, 14 of 16
 // rows: 1.22 loads per voxel).
+// FIRST: r = q itself (an infinite dual minus itself would be NaN).  A template: as a
+// flag the loads of q_prev wait for it (20 iterations at 256^3: 3.42 against 2.78 ms).
 constexpr int TS_W = 30, TS_H = 14;
 
+template <bool FIRST>
 __global__ void __launch_bounds__(32 * (TS_H + 2), 4) k_tv_step(const float *__restrict__ b, Dims d, float lam, float xmax,
                                                                 float inv12lam, float theta,
                                                                 const float *__restrict__ q, const float *__restrict__ qp,
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(32 * (TS_H + 2), 4) k_tv_step(const float *__r
     const bool h0 = a0 < d.n0 - 1, h1 = a1 < d.n1 - 1;
     auto dual = [&](size_t at) {
         const float v = q[at];
-        return fmaf(theta, v - qp[at], v);
+        return FIRST ? v : fmaf(theta, v - qp[at], v);
     };
     float r0p = 0.f, r1p = 0.f, r2p = 0.f, yp = 0.f;  // the plane below
     if (z0 > 0 && in) r2p = dual(2 * N + e - s2);
@@ -249,7 +252,8 @@ cudaError_t fgp_iterations(const float *b, const Dims &d, float lam, float xmax,
     int c = *cur, prev = *cur;
     for (int it = 0; it < iters; ++it) {
         const int next = it == 0 ? (c + 1) % 3 : 3 - c - prev;
-        k_tv_step<<<grid, dim3(32, TS_H + 2), 0, st>>>(b, d, lam, xmax, inv12, theta, q[c], q[prev], q[next], planes);
+        auto step = it == 0 ? k_tv_step<true> : k_tv_step<false>;
+        step<<<grid, dim3(32, TS_H + 2), 0, st>>>(b, d, lam, xmax, inv12, theta, q[c], q[prev], q[next], planes);
         const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
         theta = (float)((t - 1.0) / tn);
         prev = c;
