@@ -235,12 +235,18 @@ cudaError_t fgp_iterations(const float *b, const Dims &d, float lam, float xmax,
     const float inv12 = (float)(1.0 / (12.0 * (double)lam));
     // planes per block: the fewest planes read (one more than written) over full
     // waves of 4 blocks per SM
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 1;
+    }();
+    const int wave = 4 * sms;
     const int64_t cols = (int64_t)((d.n0 + TS_W - 1) / TS_W) * ((d.n1 + TS_H - 1) / TS_H);
     int planes = d.n2;
     int64_t best = INT64_MAX;
     for (int c = 1; c <= d.n2 && c <= 64; ++c) {
         const int p = (d.n2 + c - 1) / c;
-        const int64_t waves = (cols * ((d.n2 + p - 1) / p) + 152 * 4 - 1) / (152 * 4);
+        const int64_t waves = (cols * ((d.n2 + p - 1) / p) + wave - 1) / wave;
         if (waves * (p + 2) < best) {
             best = waves * (p + 2);
             planes = p;
