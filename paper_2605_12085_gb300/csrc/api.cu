@@ -358,7 +358,7 @@ extern "C" fbl_status geometry_create(const fbl_geometry_desc *desc, fbl_geometr
     // 512^3 5.13; with 8 columns and loads one sample ahead 15.7, 0.357, 5.38)
     dg.k1_cols = 4;
     dg.k1_split = 0;
-    dg.wide_rows = max_step > STRIP_MAX_STEP ? 1 : 0;
+    dg.wide_rows = max_step > COLUMN_MAX_STEP ? 2 : max_step > STRIP_MAX_STEP ? 1 : 0;
     dg.k2_vpl = backproject_default_config(dg);
     // detector rows with a crossing in (k - 1, k + 1) on one column: at most
     // floor(2 max_inv) + 1

@@ -130,7 +130,7 @@ struct DevGeom {
     float sod, sdd, inv_du;
     float hwu;                   // half width, in columns, of a voxel's column footprint
     int ntap;                    // detector rows that can touch one voxel in one column
-    int wide_rows;               // some rows cross the volume more than STRIP_MAX_STEP voxels apart
+    int wide_rows;               // rows cross the volume more than STRIP_MAX_STEP (1) or COLUMN_MAX_STEP (2) voxels apart
     // launch configuration (by the autotuner; defaults 4 / 0 / by the volume's size)
     int k1_cols;                 // projector: detector columns per block (4 or 8)
     int k1_split;                // projector plane loop: 0 plain, 1 loads one sample ahead, 2 TMA-staged bricks
@@ -222,6 +222,10 @@ constexpr int STRIP_EDGE = 8;
 // 256 voxels: columns 2.4e-7 at 1 voxel, 1.7e-7 from 1.5 on; strips 1.1e-7 at 1,
 // 1.3e-7 at 1.5, 1.5e-7 at 2, 2.1e-7 at 3, 3e-7 at 4, 8e-5 at 12, 9e-4 at 110.)
 constexpr double STRIP_MAX_STEP = 2.0;
+// Columns convert a spacing and an offset in voxels to FP32 from 32 bits in Q.24, which
+// end at 128 voxels; with rows further apart than this (and an offset of at most 2 more)
+// they convert the 64 bits.
+constexpr double COLUMN_MAX_STEP = 120.0;
 __host__ __device__ __forceinline__ bool k2_is_strips(const DevGeom &g) {
     return !g.wide_rows && (g.k2_vpl == 8 || g.k2_vpl == 16 || g.k2_vpl == 28);
 }

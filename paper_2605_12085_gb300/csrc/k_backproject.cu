@@ -45,7 +45,7 @@ constexpr int K2_LANES = 32;
 // one voxel column per warp with that many consecutive voxels per lane; 8 and 28
 // are strips with 4 or 8 voxels per lane, 16 strips with 6 (all three run as 4
 // where the geometry's rows are too far apart for strips).
-__host__ __device__ __forceinline__ int k2_vpl_of(const DevGeom &g) { return g.k2_vpl == 2 ? 2 : 4; }
+__host__ __device__ __forceinline__ int k2_vpl_of(const DevGeom &g) { return g.k2_vpl == 2 && g.wide_rows < 2 ? 2 : 4; }
 constexpr int K2_WARPS = 8;   // consecutive i per block
 
 // Packed FP32x2 arithmetic (sm_100 family): the same IEEE operation on each
@@ -187,8 +187,8 @@ __device__ __forceinline__ void column_profile(float (&acc)[VPL], float wb, cons
 
 // One block's work: voxel columns i = bx*8 .. bx*8+7 of row j, z-span bz;
 // the block's sum of squared gradient values goes to *g2_partial (if not NULL).
-// Called by every thread.
-template <int NTAP, int K2_VPL>
+// WIDE: rows too far apart for 32-bit conversions.  Called by every thread.
+template <int NTAP, int K2_VPL, bool WIDE = false>
 __device__ __forceinline__ void k2_tile(const BpArgs &a, int bx, int j, int bz, double *g2_partial) {
     constexpr int K2_KSPAN = K2_LANES * K2_VPL;
     const DevGeom &g = a.g;
@@ -229,13 +229,15 @@ __device__ __forceinline__ void k2_tile(const BpArgs &a, int bx, int j, int bz, 
             // row iv crosses plane m at q_z = 2*iv*Z + zoff (Q.40), 0 < Z < 2^40
             const long long Z = cF.h0 + (long long)m * cF.h1;
             const long long zoff = g.cz_fx - (long long)(g.nv - 1) * Z;
-            const float step = (float)(int)(Z >> 15) * kInv24;  // dq_z per row = 2Z (32-bit path)
+            // dq_z per row = 2Z (32-bit path)
+            const float step = WIDE ? (float)(Z >> 15) * kInv24 : (float)(int)(Z >> 15) * kInv24;
             const float inv = __fdividef(1.f, step);            // rows per voxel (estimate)
             const float zoff_f = g.cz - (float)(g.nv - 1) * 0.5f * step;
             // first row whose crossing lies above kfirst - 1: estimate, then one exact correction
             int lo = (int)ceilf(((float)kfirst - zoff_f) * inv - inv);
             const long long d_fx = 2LL * lo * Z + zoff - kfirst_fx;
-            float d0 = (float)(int)(d_fx >> 16) * kInv24;  // q_z(lo) - kfirst (|.| < 2 + step)
+            // q_z(lo) - kfirst (|.| < 2 + step)
+            float d0 = WIDE ? (float)(d_fx >> 16) * kInv24 : (float)(int)(d_fx >> 16) * kInv24;
             if (d0 <= -1.f) {
                 ++lo;
                 d0 += step;
@@ -276,6 +278,17 @@ template <int NTAP, int K2_VPL>
 __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 5) k2_backproject(const BpArgs a) {
     const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     k2_tile<NTAP, K2_VPL>(a, blockIdx.x, blockIdx.y, blockIdx.z, a.g2_partials ? a.g2_partials + blk : nullptr);
+}
+
+// Rows more than COLUMN_MAX_STEP voxels apart: one form for all such geometries (a larger
+// NTAP only adds tested rows), a call of its own in the batch, so that the usual tiles
+// keep their registers (as a flag in them: 1.7 % of small batches).
+__device__ __noinline__ void k2_tile_wide(const BpArgs &a, int bx, int j, int bz, double *g2_partial) {
+    k2_tile<RT_PAD, 4, true>(a, bx, j, bz, g2_partial);
+}
+__global__ void __launch_bounds__(K2_LANES *K2_WARPS) k2_backproject_wide(const __grid_constant__ BpArgs a) {
+    const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    k2_tile_wide(a, blockIdx.x, blockIdx.y, blockIdx.z, a.g2_partials ? a.g2_partials + blk : nullptr);
 }
 
 // Persistent batched backprojector: the blocks of k2_backproject of every volume
@@ -319,7 +332,8 @@ __global__ void __launch_bounds__(K2_LANES *K2_WARPS, 4) kb_backproject(const Ba
         const int j = rest % bv.g.ny;
         const int bz = rest / bv.g.ny;
         double *part = bv.partials + local;
-        if (k2_vpl_of(bv.g) == 2) k2_tile<NTAP, 2>(a, bx, j, bz, part);
+        if (bv.g.wide_rows > 1) k2_tile_wide(a, bx, j, bz, part);
+        else if (k2_vpl_of(bv.g) == 2) k2_tile<NTAP, 2>(a, bx, j, bz, part);
         else k2_tile<NTAP, 4>(a, bx, j, bz, part);
     }
     batch_leave(ctr);
@@ -409,6 +423,10 @@ cudaError_t launch_backproject(const DevGeom &g, const float *rt, const int32_t 
     dim3 block(K2_LANES, K2_WARPS);
     const dim3 grid = k2_grid(g);
     if (k2_is_strips(g)) return launch_strips(a, grid, strip_zp(g.k2_vpl, g.nz), st);
+    if (g.wide_rows > 1) {
+        k2_backproject_wide<<<grid, block, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     const int vpl = k2_vpl_of(g);
     switch (g.ntap) {  // rows per voxel and column, fixed per geometry (<= RT_PAD)
         case 1: launch_k2<1>(vpl, grid, block, st, a); break;

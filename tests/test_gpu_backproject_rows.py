@@ -34,7 +34,7 @@ def _check(G, g, rng):
 
 
 @pytest.mark.parametrize("vpl", [2, 4, 16, 28])
-@pytest.mark.parametrize("spacing", [1.9, 2.1, 4, 9, 16, 40, 100])
+@pytest.mark.parametrize("spacing", [1.9, 2.1, 4, 9, 16, 40, 100, 119, 121, 200, 500])
 def test_rows_far_apart_match_oracle(spacing, vpl):
     import paper_2605_12085_gb300 as fbl
     g = _geom(spacing)
@@ -50,10 +50,11 @@ def test_default_configuration_of_a_volume_that_fills_the_gpu(spacing):
     _check(fbl.geometry_create(g), g, np.random.default_rng(1))
 
 
-def test_batch_with_rows_far_apart_equals_single_solvers():
+@pytest.mark.parametrize("spacing", [20, 200])
+def test_batch_with_rows_far_apart_equals_single_solvers(spacing):
     # the volume asks for strips and runs in columns, beside one that runs in strips
     import paper_2605_12085_gb300 as fbl
-    gs = [_geom(20, nx=12, ny=11, nz=70, views=8), _geom(1.2, nx=9, ny=14, nz=40, views=6)]
+    gs = [_geom(spacing, nx=12, ny=11, nz=70, views=8), _geom(1.2, nx=9, ny=14, nz=40, views=6)]
     rng = np.random.default_rng(5)
     Gs, bs, ps = [], [], []
     for q, g in enumerate(gs):
