@@ -33,7 +33,10 @@
 // where the weight may end), and one coalesced load and half a packed FMA per
 // row: two rows where rows are more than a voxel apart, three down to 2/3 of a
 // voxel, four down to 1/2 (uniform over the warp), with no chain from one voxel
-// to the next.
+// to the next.  The position is a fraction of a row, so rows are at most
+// STRIP_MAX_STEP voxels apart here.  The rows taken in beside a voxel have weight
+// 0; where some residual is infinite or NaN, an instantiation that leaves them out
+// runs instead (launch_weight's flag).
 //
 // Measured (40 views at 512^3, 768^2; CUDA events): 8.23 ms for the 2 x 2 groups
 // at 44.5 warp instructions per 32 voxel-views; 7.58 with strips and their sums in
@@ -559,11 +562,12 @@ __host__ __device__ __forceinline__ int strip_parts(const DevGeom &g, int n_sel)
     const size_t parts = (bytes + STRIP_BYTES - 1) / STRIP_BYTES;
     return (int)(parts < (size_t)n_sel ? parts : (size_t)n_sel);
 }
-// The rows and views of part p of n_sel.
-__host__ __device__ __forceinline__ void strip_part(BpArgs &a, const float *rt, const int32_t *views, int n_sel, int p,
-                                                    int parts) {
+// The rows and views of part p of n_sel (g apart from a: a block's copy of it is still
+// being staged when its first part is set).
+__host__ __device__ __forceinline__ void strip_part(BpArgs &a, const DevGeom &g, const float *rt, const int32_t *views,
+                                                    int n_sel, int p, int parts) {
     const int s0 = (int)((int64_t)n_sel * p / parts), s1 = (int)((int64_t)n_sel * (p + 1) / parts);
-    a.rt = rt + (size_t)s0 * a.g.nu * rt_pitch(a.g.nv);
+    a.rt = rt + (size_t)s0 * g.nu * rt_pitch(g.nv);
     a.views = views + s0;
     a.n_sel = s1 - s0;
     a.more = p > 0;
@@ -609,7 +613,7 @@ __global__ void __launch_bounds__(32 * KBS_WARPS, KBS_BLOCKS) kb_strips(const Ba
 #pragma unroll 1
         for (int p = 0; p < parts; ++p) {
             if (p > 0) __syncthreads();  // the last part's arguments and sums
-            if (tid == 0) strip_part(sa, bv.rt, bv.views, bv.N_t, p, parts);
+            if (tid == 0) strip_part(sa, bv.g, bv.rt, bv.views, bv.N_t, p, parts);
             __syncthreads();
             double *part = a.last ? bv.partials + local : nullptr;
             switch (strip_zp(bv.g.k2_vpl, bv.g.nz)) {
@@ -647,7 +651,7 @@ cudaError_t launch_strips(const BpArgs &a, dim3 grid, int zp, cudaStream_t st) {
     const int parts = strip_parts(a.g, a.n_sel);
     for (int p = 0; p < parts; ++p) {
         BpArgs b = a;
-        strip_part(b, a.rt, a.views, a.n_sel, p, parts);
+        strip_part(b, a.g, a.rt, a.views, a.n_sel, p, parts);
         if (!b.last) b.g2_partials = nullptr;
         k<<<grid, 32 * STRIP_EDGE, 0, st>>>(b);
     }
