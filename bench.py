@@ -888,8 +888,9 @@ def alu_roofline(kernel, ops_per_sample, samples, avg_ms, algorithmic_bytes, clk
 
 def fblisa_iteration_record(fbl, G, g, wl, b, device, steps, warmup, peaks):
     """One FB-LISA iteration (Steps 2a-2d, host loop, FP32) on the workload's
-    40-view mini-batches: GUPS over the work an iteration does (every forward
-    projection N_t nu nv N samples, the backprojection N_t N^3 voxel-views),
+    40-view mini-batches: GUPS over the work an iteration completes (the residual
+    projection and the accepted trial's objective, N_t nu nv N samples each, and the
+    backprojection, N_t N^3 voxel-views; rejected trials end early),
     per-kernel CUDA-event times recorded by the library on the launching
     stream, and the rooflines of the residual projection (K1; a trial's objective
     may end early), the gradient backprojection (K2) and the prox (K3)."""

@@ -32,6 +32,12 @@
  * Streams: "stream" is a cudaStream_t (NULL = the legacy default stream).
  *   project/backproject enqueue work and return; calls with host outputs
  *   (scalars or host volumes) return after the results are on the host.
+ * Memory: the calls' scratch comes from a stream-ordered pool of the library, one
+ *   per device; while a geometry lives on the device the pool keeps up to 4 GiB
+ *   of what was used between calls.  Other allocations of the same process get
+ *   its idle memory when the device is full, other processes do not; it goes back
+ *   with the last geometry.  Captured calls, and calls without a geometry while
+ *   none lives, use the device's default pool.
  * Device: objects are bound to the CUDA device current at creation; calls
  *   must be made with that device current.
  * Errors: calls return a status and never throw; the message of the last
@@ -179,7 +185,8 @@ typedef struct {
  * geometry_autotune -- time the projector and backprojector launch
  * configurations on this geometry (n_sel views spread over the orbit, storage
  * x_dtype) and keep the fastest for later calls on g.  Results do not depend
- * on the configuration beyond FP32 summation order.  Not safe to call while
+ * on the configuration beyond FP32 rounding (the order of sums, and in the
+ * backprojector the form of the weights).  Not safe to call while
  * other calls use g.  report may be NULL.
  */
 FBL_API fbl_status geometry_autotune(fbl_geometry *g, int32_t x_dtype, int32_t n_sel, void *stream,
@@ -213,7 +220,8 @@ FBL_API fbl_status project(const fbl_geometry *g, const void *x, int32_t x_dtype
  * backproject -- x = A_N^T y (or x += A_N^T y when accumulate != 0), the
  * exact transpose of project, needed by grad f_N in Step 2b of Algorithm 1.
  * y: [n_sel][nv][nu] of y_dtype (may be NULL when n_sel == 0); x: [nz][ny][nx]
- * float32 (zeroed when n_sel == 0 and accumulate == 0).
+ * float32 (zeroed when n_sel == 0 and accumulate == 0).  An infinite or NaN pixel
+ * makes the voxels its ray touches infinite or NaN, and no others.
  */
 FBL_API fbl_status backproject(const fbl_geometry *g, const void *y, int32_t y_dtype,
                        const int32_t *views, int32_t n_sel, float *x, int32_t accumulate,

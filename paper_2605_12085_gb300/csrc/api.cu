@@ -74,7 +74,8 @@ fbl_status check_device(int want) {
 // lives on it.  The device's default pool gives its memory back at every
 // synchronisation, so that a call after one maps its scratch anew (256^3, 20
 // views: 859 us for a first backproject() against 409 us for the next); this pool
-// keeps up to kPoolKeep between calls and gives it back with the last geometry.
+// keeps up to kPoolKeep between calls and gives it back with the last geometry.  (Other
+// allocations of the process get what is idle in it where the device is full.)
 constexpr uint64_t kPoolKeep = uint64_t(4) << 30;
 constexpr int kPoolDevices = 64;
 struct ScratchPool {

@@ -174,10 +174,12 @@ int project_num_partials(const DevGeom &g, int n_sel);
 // views, 2 us a trial.)
 bool project_may_stop(const DevGeom &g, int n_sel);
 // The same for a batch whose trial objectives have `tiles` blocks in all: more than
-// eight waves.  Forming the limit costs a batch about 2 us a trial round (passes over
-// 4 volumes of 20^3..41^3: 2.48 ms with the limit, 2.40 without; 12 of 24^3..60^3: 4.86
-// and 4.74; 16 of 24^3..80^3: 9.58 and 9.48, with the line at 1, 2 or 4 waves 9.57 to
-// 9.58), larger batches gain (16 of 96^3..320^3 have far more).
+// eight waves.  Forming the limit costs a batch about 2 us a trial round.  12 iterations
+// with the limit always / never in force, the first epoch (more rejected trials) and a
+// later one, ms, by waves: 0.4 (4 volumes of 20^3..41^3) 2.48/2.41 and 2.16/2.12; 4.5
+// (16 of 24^3..80^3) 9.40/9.27 and 8.41/8.28; 5.2 11.20/11.30 and 10.47/10.33; 9.3
+// (16 of 60^3..100^3) 18.26/18.36 and 16.93/16.79; 17.5 31.8/33.5 and 30.5/30.3; 28
+// (16 of 96^3..160^3) 53.1/58.5 and 53.9/53.8; 43 85.8/100.1 and 89.4/90.8.
 constexpr int BATCH_STOP_WAVES = 8;
 bool batch_may_stop(int cols, int64_t tiles);
 

@@ -9,8 +9,8 @@
 // two adjacent rows b0, b0+1 of the z-innermost volume layout over a run of
 // consecutive k: about five 32-byte sectors per load instead of one sector
 // per lane.  Both ray families read the same volume copy with their own
-// plane and in-plane strides.  A block is 8 columns of one view; the grid runs the 32-row
-// bands slowest, so the blocks resident together cover every view of the
+// plane and in-plane strides.  A block is 4 or 8 columns of one view (k1_cols; 4 unless
+// tuned); the grid runs the 32-row bands slowest, so the blocks resident together cover every view of the
 // batch for one band of rows and share a z-slab of the volume in L2.
 //
 // Arithmetic.  Per-ray constants come from the geometry's column tables (FP64
