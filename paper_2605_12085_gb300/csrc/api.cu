@@ -517,15 +517,18 @@ fbl_status upload_views(const int32_t *views, int32_t n, AsyncBuf &buf, cudaStre
     return FBL_OK;
 }
 
-// The same with a word behind the list that is 0 (in the same copy, but for a
-// captured call, whose copy reads the caller's list when the graph runs).
+// The same with a word behind the list that is 0: in the same copy for lists of
+// ordinary length, but for a captured call, whose copy reads the caller's list when
+// the graph runs.
 fbl_status upload_views_and_zero(const int32_t *views, int32_t n, AsyncBuf &buf, cudaStream_t st) {
+    constexpr int32_t kList = 2048;
     CK(buf.alloc(((size_t)n + 1) * sizeof(int32_t), st), "view list");
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-        std::vector<int32_t> list(views, views + n);
-        list.push_back(0);
-        CK(cudaMemcpyAsync(buf.p, list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st),
+    if (n < kList && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        int32_t list[kList];
+        std::memcpy(list, views, (size_t)n * sizeof(int32_t));
+        list[n] = 0;
+        CK(cudaMemcpyAsync(buf.p, list, ((size_t)n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st),
            "view list copy");
         return FBL_OK;
     }

@@ -33,3 +33,25 @@ def test_nonfinite_pixels_reach_the_voxels_of_their_rays(dv, nv, vpl):
     free = weight == 0
     assert np.isfinite(got[free]).all()
     assert rel_l2(got[free], oracle.backproject(g, clean.astype(np.float64), range(4))[free]) <= 1e-5
+
+
+@pytest.mark.parametrize("n", [1, 2047, 2048, 2600])
+def test_view_lists_of_any_length(n):
+    # the word that notes such pixels stands behind the view list: in one copy with it below
+    # 2048 views, cleared by itself above; repeated views (sums of n FP32 terms: 1e-5)
+    import paper_2605_12085_gb300 as fbl
+    g = synth.Geometry(nx=9, ny=8, nz=12, vx=1.0, vy=1.0, vz=1.0, n_views=5, sod=400.0, sdd=700.0, nu=12, nv=16, du=1.7, dv=1.5)
+    G = fbl.geometry_create(g)
+    fbl.geometry_set_launch(G, 4, 0, 28)
+    rng = np.random.default_rng(n)
+    views = [int(v) for v in rng.integers(0, 5, n)]
+    y = rng.standard_normal((n, 16, 12)).astype(np.float32)
+    ref = oracle.backproject(g, y.astype(np.float64), views)
+    assert rel_l2(host(fbl.backproject(G, cuda(y), views)), ref) <= 1e-5
+    y[n - 1, 8, 6] = np.nan
+    hit = np.zeros(y.shape)
+    hit[n - 1, 8, 6] = 1.0
+    weight = oracle.backproject(g, hit, views)
+    got = host(fbl.backproject(G, cuda(y), views))
+    assert np.isnan(got[weight > 1e-6]).all() and np.isfinite(got[weight == 0]).all()
+    assert rel_l2(host(fbl.backproject(G, cuda(np.nan_to_num(y)), views))[weight == 0], ref[weight == 0]) <= 1e-5
